@@ -69,8 +69,12 @@ DF_OPS = 8 * (12 * 8 + 6 * (2 * 3 + 2 * 11) + 12 * 4 * 11 + 24 * 8) + 8 * 30 + 1
 # lane-pair sums (12 x (2 x 2 x 29 + 8)) and 30 for their bounds; U + kappa H and the stores.
 DF_OPS_GRID = 8 * (12 * 8 + 6 * (2 * 2 * 14 + 8) + 16 + 24 * 8) + 8 * 30 \
     + 12 * (2 * 2 * 29 + 8) + 30 + 24 * 11 + 24 * 3
-# FP64-pipe operations per site and RHS of the FP32-lane form of the FP64 stencils
-# (csrc/dslash_x3.cu, wd_set_apply_form 1): the spin projections (8 hops x 12 real FMAs), joining
+# 32x32+64-bit multiply-adds per site and RHS of the fixed-point FP64 stencils (csrc/dslash_fx.cu,
+# wd_set_apply_form 1): a complex product takes three real ones of three multiply-adds each; the 8
+# hops make 2 spins x 9 of them, the two 6x6 site blocks 72.
+FX_MULS = 9 * (8 * 18 + 72)
+# FP64-pipe and FP32-lane operations per site and RHS of the same stencils with the hopping sums in
+# exact FP32 grid sums (the form before the fixed-point one, kept for comparisons): the spin projections (8 hops x 12 real FMAs), joining
 # the three levels of the 24 hopping sums (2 adds each), the 24 final FMAs with kappa, and the two
 # Hermitian 6x6 site blocks (6 real x complex products and 15 complex entries used twice, 4 FMAs per
 # complex product: 2 x (12 + 120)).  The hopping products themselves run on the FP32 lanes: 288
@@ -192,7 +196,7 @@ KERNEL_SOURCES = {
     ("dslash_jacobi_lp", "df"): ["sweep_df.cu", "common.cuh", "elem.cuh", "internal.h"],
     ("dslash_jacobi_lp", "fp32"): ["sweep_lp.cuh", "sweep_f32.cu", "sweep_lp.cu", "common.cuh",
                                    "elem.cuh", "internal.h"],
-    ("dslash_apply", "fp64"): ["dslash_x3.cu", "dslash.cu", "common.cuh", "spin.cuh", "internal.h"],
+    ("dslash_apply", "fp64"): ["dslash_fx.cu", "fixed.cuh", "dslash.cu", "common.cuh", "internal.h"],
 }
 
 
@@ -881,8 +885,8 @@ def main():
         n, ms = prof.get(cls, (0, 0.0))
         if not n:
             continue
-        # the FP32-lane form launches an exponent pre-pass with each FP64 stencil
-        per_launch = 2 if stencil_form == 1 and cls in ("dslash_apply", "dslash_jacobi") else 1
+        # the fixed-point form copies a product's operand into its own form first
+        per_launch = 2 if stencil_form == 1 and cls == "dslash_apply" else 1
         n //= per_launch
         avg_s = ms / n / 1e3
         kprec = sweep_prec if cls == "dslash_jacobi_lp" else "fp64"
@@ -910,17 +914,14 @@ def main():
                 "unit": "T FP32 lane ops/s", "frac": round(tops / alu["fp32_lane_tops"], 4),
                 "peak_source": alu_source + " x 128 FP32 lanes", "fp32_ops_per_site_rhs": ops}
         elif not f32 and stencil_form == 1:
-            # the FP32-lane form: FP64 pipe and FP32 lanes both carry work; the FP64 pipe is the
-            # busier one (ncu)
-            ops64 = X3_FP64_OPS * V * L_RHS / avg_s / 1e12
-            ops32 = X3_FP32_OPS * V * L_RHS / avg_s / 1e12
+            # the fixed-point form: the multiplier pipe, one quarter of a warp per clock and quadrant
+            muls = FX_MULS * V * L_RHS / avg_s / 1e12
+            peak = sm_count * 32 * clock_mhz * 1e6 / 1e12
             fig["binding_roofline"] = {
-                "bound": "alu", "achieved": round(ops64, 4), "peak": round(alu["fp64_tflops"] / 2, 4),
-                "unit": "T FP64-pipe ops/s", "frac": round(ops64 / (alu["fp64_tflops"] / 2), 4),
-                "peak_source": alu_source + " x 2 FP64 lanes/clk", "fp64_ops_per_site_rhs": X3_FP64_OPS,
-                "fp32_lane_ops_per_site_rhs": X3_FP32_OPS,
-                "fp32_lane_frac": round(ops32 / alu["fp32_lane_tops"], 4),
-                "form": "hopping sums on the FP32 lanes (wd_set_apply_form 1)"}
+                "bound": "alu", "achieved": round(muls, 4), "peak": round(peak, 4),
+                "unit": "T 32x32+64-bit multiply-adds/s", "frac": round(muls / peak, 4),
+                "peak_source": alu_source + " x 32 lanes/clk", "multiply_adds_per_site_rhs": FX_MULS,
+                "form": "64-bit fixed point (wd_set_apply_form 1)"}
         elif not f32:
             fig["binding_roofline"] = {
                 "bound": "alu", "achieved": round(tflops, 4), "peak": round(alu["fp64_tflops"], 4),

@@ -306,11 +306,13 @@ int wd_set_link_reals(wd_ctx* ctx, int reals);
 /* Form of the FP64 stencil Y = A X, R = B - A X and of the FP64 Jacobi sweep (Eq. (1), Sec. 2),
  * which carry the outer method's products W = AF, Y = AG, the true residual and precision 0's
  * preconditioner.  1 (the default for links whose rows and columns have norm <= 1 + 1e-6, so
- * unitary links): the hopping sums run on the FP32 lanes, every operand cut exactly into three
- * FP32 numbers and the products summed exactly on fixed grids, so that the hopping term is
- * exact to ~2^-52 of its bound before one FP64 rounding; the site blocks, the spin projection
- * and the final combination stay FP64.  It is as accurate as FP64 arithmetic and about twice as
- * fast on GB300, whose FP64 pipe issues two lanes per clock per SM.  0: every operation on the
+ * unitary links): 64-bit fixed point on the integer pipes -- spinors as integers of 58 bits with one
+ * exponent per (site, right-hand side), the operator as integers of 60 bits, exact sums, one rounding
+ * per hop to 2^-58 of the largest entry around the site and one to FP64.  It is more accurate than
+ * FP64 arithmetic and over four times as fast on GB300, whose FP64 pipe issues two lanes per clock per
+ * SM.  A product with A copies its operand into a block of this form, which the context allocates at
+ * the first product with a given L; when there is no room for it, or while the stream is being
+ * captured before the block exists, the product runs as with 0.  0: every operation on the
  * FP64 pipe.  Asking for 1 with other links is WD_EINVAL.  wd_get_apply_form returns the form
  * (-1 for a NULL ctx). */
 int wd_set_apply_form(wd_ctx* ctx, int form);

@@ -449,7 +449,7 @@ def wd_copy_residual(ctx: Context, R):
 
 
 def wd_set_apply_form(ctx: Context, form: int) -> None:
-    """Form of the FP64 stencils: 1 = hopping sums exact on the FP32 lanes (unitary links), 0 = FP64 pipe."""
+    """Form of the FP64 stencils: 1 = 64-bit fixed point (unitary links), 0 = FP64 pipe."""
     _check(lib().wd_set_apply_form(ctx.handle, int(form)))
 
 

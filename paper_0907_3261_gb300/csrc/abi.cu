@@ -119,6 +119,8 @@ struct wd_ctx {
   DevBuf stage_in, stage_out;
   // low-precision preconditioner blocks: U and two sweep buffers (sized for FP32 elements)
   DevBuf blk32[3];
+  // the copy of a product's operand in the fixed-point stencil's form (one block)
+  DevBuf field;
   // autotuned tile of the low-precision sweep per storage (LP_F32, LP_BF16, LP_DF) and L: RHS per
   // thread, threads per CTA, min CTAs per SM, shared-memory staging
   int tile_r[3][WD_LMAX + 1] = {};
@@ -251,6 +253,30 @@ int ensure_workspace(wd_ctx* c, int L) {
   return WD_OK;
 }
 
+// The block for the fixed-point stencil's copy of its operand, allocated at the first product with an L
+// (grown, never shrunk).  Null -- the product then runs on the FP64 pipe, which needs no
+// memory -- when the form is not in use, when the device has no room for the block, or when it would
+// have to be allocated while `s` is being captured.
+void* field_block(wd_ctx* c, int L, cudaStream_t s) {
+  if (c->op.apply_form != 1) return nullptr;
+  const size_t bytes = block_bytes(c, L);
+  if (c->field.bytes < bytes) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    c->field.release();
+    if (cudaMalloc(&c->field.p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      c->field.p = nullptr;
+      return nullptr;
+    }
+    c->field.bytes = bytes;
+  }
+  return c->field.p;
+}
+
 // Picks the low-precision sweep's tile (RHS per thread, threads per CTA, min CTAs per SM, staging) for this
 // lattice, storage and L by timing every candidate on the context's blocks (zeroed first); the
 // winner is kept in the context.
@@ -371,7 +397,7 @@ long long slice_sites(const wd_ctx* c) {
 constexpr int DOM_REDUCE_DOUBLES = 2 * WD_LMAX * WD_LMAX + 2 * WD_LMAX;
 
 int dom_staging(wd_ctx* c, int L) {
-  const size_t slice = (size_t)slice_sites(c) * 12 * L * 16;
+  const size_t slice = (size_t)slice_sites(c) * L * (12 * 16 + sizeof(short)) + 16;
   const size_t need = 4 * slice + DOM_REDUCE_DOUBLES * sizeof(double);
   if (c->dom_host_bytes >= need) return WD_OK;
   if (c->dom_host) cudaFreeHost(c->dom_host);
@@ -383,25 +409,31 @@ int dom_staging(wd_ctx* c, int L) {
 }
 
 // Fills the two halo slices of a block (N x L, site-major, the context's extended slab) from the
-// neighbouring ranks: the first and last interior slices go out, the received slices come in.
-int halo_exchange(wd_ctx* c, double* blk, int L, cudaStream_t s) {
+// neighbouring ranks: the first and last interior slices go out, the received slices come in.  exps:
+// the exponents of a block in the fixed-point form, whose slices travel behind the block's.
+int halo_exchange(wd_ctx* c, void* blk, int L, cudaStream_t s, short* exps = nullptr) {
   if (!c->dom_on) return WD_OK;
   CHECK(dom_staging(c, L));
   const long long Vs = slice_sites(c), V = c->op.g.V;
-  const size_t slice = (size_t)Vs * 12 * L * 16;
-  const size_t per_site = (size_t)12 * L * 2;   // doubles
+  const size_t site = (size_t)12 * L * 16, esite = (size_t)L * sizeof(short);   // bytes per site
+  const size_t body = (size_t)Vs * site, slice = body + (exps ? Vs * esite : 0);
   char* h = static_cast<char*>(c->dom_host);
-  CU(cudaMemcpyAsync(h, blk + (size_t)Vs * per_site, slice, cudaMemcpyDeviceToHost, s));
-  CU(cudaMemcpyAsync(h + slice, blk + (size_t)(V - 2 * Vs) * per_site, slice,
-                     cudaMemcpyDeviceToHost, s));
+  char* d = static_cast<char*>(blk);
+  char* e = reinterpret_cast<char*>(exps);
+  const long long from[2] = {Vs, V - 2 * Vs}, to[2] = {0, V - Vs};
+  for (int k = 0; k < 2; ++k) {
+    CU(cudaMemcpyAsync(h + k * slice, d + from[k] * site, body, cudaMemcpyDeviceToHost, s));
+    if (e) CU(cudaMemcpyAsync(h + k * slice + body, e + from[k] * esite, Vs * esite, cudaMemcpyDeviceToHost, s));
+  }
   CU(cudaStreamSynchronize(s));
   if (c->dom.exchange(h, h + slice, h + 2 * slice, h + 3 * slice, slice, c->dom.user) != 0) {
     set_err("wd_domain.exchange failed");
     return WD_ECUDA;
   }
-  CU(cudaMemcpyAsync(blk, h + 2 * slice, slice, cudaMemcpyHostToDevice, s));
-  CU(cudaMemcpyAsync(blk + (size_t)(V - Vs) * per_site, h + 3 * slice, slice,
-                     cudaMemcpyHostToDevice, s));
+  for (int k = 0; k < 2; ++k) {
+    CU(cudaMemcpyAsync(d + to[k] * site, h + (2 + k) * slice, body, cudaMemcpyHostToDevice, s));
+    if (e) CU(cudaMemcpyAsync(e + to[k] * esite, h + (2 + k) * slice + body, Vs * esite, cudaMemcpyHostToDevice, s));
+  }
   return WD_OK;
 }
 
@@ -497,12 +529,23 @@ int precondition(wd_ctx* c, const double* R, double* a, double* b, double** res,
     }
     return WD_OK;
   }
-  LAUNCH(WD_K_SITE_INV, 1, launch_site_inverse_f64(op, R, a, L, s));
   double* cur = a;
   double* nxt = b;
+  const bool fields = op.apply_form == 1 && j >= 2;    // the iterates in fixed point up to the last sweep
+  if (fields)
+    LAUNCH(WD_K_SITE_INV, 1, launch_first_fx(op, R, a, 0, L, s));
+  else
+    LAUNCH(WD_K_SITE_INV, 1, launch_site_inverse_f64(op, R, a, L, s));
   for (int i = 1; i < j; ++i) {
-    CHECK(halo_exchange(c, cur, L, s));
-    LAUNCH(WD_K_JACOBI, stencil_kernels(op), launch_jacobi_f64(op, cur, R, nxt, L, s));
+    const int slot = (i - 1) & 1;
+    CHECK(halo_exchange(c, cur, L, s, fields ? op.fx_exp(slot) : nullptr));
+    if (fields) {
+      const bool last = i == j - 1;
+      LAUNCH(WD_K_JACOBI, 1,
+             launch_sweep_fx(op, cur, slot, R, last ? nullptr : nxt, last ? nxt : nullptr, L, s));
+    } else {
+      LAUNCH(WD_K_JACOBI, 1, launch_jacobi_f64(op, cur, R, nxt, L, s));
+    }
     if (hop_count) ++*hop_count;
     double* t = cur;
     cur = nxt;
@@ -561,11 +604,12 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
   double* pT = c->blk[B_T].d();
   double2* part = static_cast<double2*>(c->part.p);
   SolverState* st = c->st;
+  void* const field = field_block(c, L, s);
   CU(cudaMemsetAsync(&st->status, 0, sizeof(int), s));
 
   // R_0 = B - A X_0;  P_0 = R_0;  R~_0 = R_0
   CHECK(halo_exchange(c, X, L, s));
-  LAUNCH(WD_K_RESID, stencil_kernels(op), launch_resid_f64(op, X, B, R, L, s));
+  LAUNCH(WD_K_RESID, stencil_kernels(op, field), launch_resid_f64(op, X, B, R, field, L, s));
   ++*hop_count;
   LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(P, R, bytes, cudaMemcpyDeviceToDevice, s));
   LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(Rt, R, bytes, cudaMemcpyDeviceToDevice, s));
@@ -584,7 +628,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
   CHECK(precondition(c, R, pF, pT, &res, L, j, precision, hop_count, s));
   if (res != pF) { pT = pF; pF = res; }
   CHECK(halo_exchange(c, pF, L, s));
-  LAUNCH(WD_K_APPLY, stencil_kernels(op), launch_apply_f64(op, pF, W, L, s));
+  LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, pF, W, field, L, s));
   ++*hop_count;
   LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(V, W, bytes, cudaMemcpyDeviceToDevice, s));
   LAUNCH(WD_K_TRACE, 2, launch_traces(in(W), in(R), L, rows, part, st, s));
@@ -603,7 +647,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
     CHECK(precondition(c, U, pG, pT, &res, L, j, precision, hop_count, s));   // G_k = M U_k
     if (res != pG) { pT = pG; pG = res; }
     CHECK(halo_exchange(c, pG, L, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op), launch_apply_f64(op, pG, Y, L, s));                  // Y_k = A G_k
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, pG, Y, field, L, s));                  // Y_k = A G_k
     ++*hop_count;
     LAUNCH(WD_K_UPDATE_XR, 2, launch_update_xr(in(X), cin(pF), cin(pG), in(R), cin(W), cin(Y), cin(Rt), L, rows, part, st, s, df));   // X_{k+1}, R_{k+1}
     CHECK(dom_sum(c, st->rtr_new, 2 * L * L, s));
@@ -621,7 +665,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
     CHECK(precondition(c, R, pF, pT, &res, L, j, precision, hop_count, s));   // F_{k+1} = M R_{k+1}
     if (res != pF) { pT = pF; pF = res; }
     CHECK(halo_exchange(c, pF, L, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op), launch_apply_f64(op, pF, W, L, s));                  // W_{k+1} = A F_{k+1}
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, pF, W, field, L, s));                  // W_{k+1} = A F_{k+1}
     ++*hop_count;
     LAUNCH(WD_K_TRACE, 2, launch_traces(in(W), in(R), L, rows, part, st, s));  // Tr[W^H R], Tr[W^H W]
     CHECK(dom_sum(c, &st->trwr, 3, s));
@@ -690,8 +734,12 @@ void wd_destroy(wd_ctx* c) {
   cudaFree(c->op.clov_bound32);
   cudaFree(c->op.links32s);
   cudaFree(c->op.clov_inv32s);
-  cudaFree(c->op.links_x3);
-  cudaFree(c->op.xexp);
+  cudaFree(c->op.fx_links);
+  cudaFree(c->op.fx_clov);
+  cudaFree(c->op.fx_cinv);
+  cudaFree(c->op.fx_nb);
+  cudaFree(c->op.fx_exps);
+  c->field.release();
   for (auto& b : c->blk) b.release();
   for (auto& b : c->blk32) b.release();
   c->part.release();
@@ -739,10 +787,14 @@ static int create_impl(wd_ctx* c, const void* links, const int dims[4], cudaStre
     set_err("a 6x6 clover block A_D is singular for kappa=%g c_SW=%g", op.kappa, op.csw);
     return WD_BREAKDOWN;
   }
-  if (op.links_unitary) {   // the FP32-lane form of the FP64 stencil (its bounds need unitary links)
-    CU(cudaMalloc(&op.links_x3, V * 4 * 27 * sizeof(float4)));
-    CU(cudaMalloc(&op.xexp, V * WD_LMAX * sizeof(int)));
-    CU(launch_link_split(op, s));
+  if (op.links_unitary) {   // the fixed-point form of the FP64 stencil (its bounds need unitary links)
+    CU(cudaMalloc(&op.fx_links, V * FX_WSTR * sizeof(int4)));
+    CU(cudaMalloc(&op.fx_clov, V * FX_DSTR * sizeof(int4)));
+    CU(cudaMalloc(&op.fx_cinv, V * FX_DSTR * sizeof(int4)));
+    CU(cudaMalloc(&op.fx_nb, V * 2 * sizeof(int4)));
+    CU(cudaMalloc(&op.fx_exps, 3 * V * WD_LMAX * sizeof(short)));
+    op.fx_ek = fx_link_exponent(op.kappa);
+    CU(launch_fx_tables(op, s));
     CU(cudaStreamSynchronize(s));
     op.apply_form = 1;
   }
@@ -896,8 +948,8 @@ int wd_set_link_reals(wd_ctx* c, int reals) {
 int wd_set_apply_form(wd_ctx* c, int form) {
   if (!c) { set_err("ctx is NULL"); return WD_EINVAL; }
   if (form != 0 && form != 1) { set_err("stencil form %d not in {0, 1}", form); return WD_EINVAL; }
-  if (form == 1 && !c->op.links_x3) {
-    set_err("the FP32-lane stencil needs links whose rows and columns have norm <= 1 + %g", LINK12_TOL);
+  if (form == 1 && !c->op.fx_links) {
+    set_err("the fixed-point stencil needs links whose rows and columns have norm <= 1 + %g", LINK12_TOL);
     return WD_EINVAL;
   }
   c->op.apply_form = form;
@@ -948,7 +1000,8 @@ int wd_apply(wd_ctx* c, const void* X, void* Y, int L, void* stream) {
     xd = c->stage_in.d();
     CHECK(halo_exchange(c, c->stage_in.d(), L, s));
   }
-  LAUNCH(WD_K_APPLY, stencil_kernels(c->op), launch_apply_f64(c->op, xd, yd, L, s));
+  void* field = field_block(c, L, s);
+  LAUNCH(WD_K_APPLY, stencil_kernels(c->op, field), launch_apply_f64(c->op, xd, yd, field, L, s));
   if (!y_dev) CU(cudaMemcpyAsync(Y, yd, bytes, cudaMemcpyDeviceToHost, s));
   if (staged_x || !y_dev) CU(cudaStreamSynchronize(s));
   harvest(c);
@@ -1171,8 +1224,9 @@ int bbicggr_solve(wd_ctx* c, const void* B, void* X, int L, int j, double tol,
     if (rr.status == RUN_STALLED) rr.status = WD_NOT_CONVERGED;
     // true residual ||b_i - A x_i|| / ||b_i||
     double* T = c->blk[B_T].d();
+    void* const field = field_block(c, L, s);
     CHECK(halo_exchange(c, Xd, L, s));
-    LAUNCH(WD_K_RESID, stencil_kernels(c->op), launch_resid_f64(c->op, Xd, Bd, T, L, s));
+    LAUNCH(WD_K_RESID, stencil_kernels(c->op, field), launch_resid_f64(c->op, Xd, Bd, T, field, L, s));
     ++hops;
     double t2[WD_LMAX];
     LAUNCH(WD_K_COLNORM, 2, launch_colnorms(T + off, L, rows, static_cast<double2*>(c->part.p), c->bnorm2_dev + WD_LMAX, s));
@@ -1411,6 +1465,7 @@ int build_run(wd_ctx* c, const JobPtrs& jp, int mode, bool df, bool restore, cud
   SolverState* st = c->st;
   GraphCtl* g = static_cast<GraphCtl*>(c->gctl);
   double* hist = c->ghist;
+  void* const field = c->op.apply_form == 1 ? c->field.p : nullptr;
 
   cudaGraphConditionalHandle hloop;
   CU(cudaGraphConditionalHandleCreate(&hloop, RB, 0, 0));
@@ -1423,14 +1478,14 @@ int build_run(wd_ctx* c, const JobPtrs& jp, int mode, bool df, bool restore, cud
       CU(cudaGetLastError());
     }
     CU(cudaMemsetAsync(&st->status, 0, sizeof(int), s));
-    LAUNCH(WD_K_RESID, stencil_kernels(op), launch_resid_f64(op, jp.X, jp.B, R, L, s));
+    LAUNCH(WD_K_RESID, stencil_kernels(op, field), launch_resid_f64(op, jp.X, jp.B, R, field, L, s));
     LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(P, R, bytes, cudaMemcpyDeviceToDevice, s));
     LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(Rt, R, bytes, cudaMemcpyDeviceToDevice, s));
     LAUNCH(WD_K_GRAM, 2, launch_gram(Rt, R, L, rows, part, st, GRAM_RTR, true, s));
     graph_init_check<<<1, 32, 0, s>>>(st, g, hist, hloop);
     CU(cudaGetLastError());
     CHECK(precondition_into(c, R, F, T, L, j, mode, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op), launch_apply_f64(op, F, W, L, s));
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, F, W, field, L, s));
     LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(V, W, bytes, cudaMemcpyDeviceToDevice, s));
     LAUNCH(WD_K_TRACE, 2, launch_traces(W, R, L, rows, part, st, s));
     LAUNCH(WD_K_GRAM, 2, launch_gram(Rt, V, L, rows, part, st, GRAM_RTV, false, s));
@@ -1451,7 +1506,7 @@ int build_run(wd_ctx* c, const JobPtrs& jp, int mode, bool df, bool restore, cud
     LAUNCH(WD_K_SOLVE_LL, 1, launch_solve_alpha(st, L, s));
     LAUNCH(WD_K_UPDATE_U, 1, launch_update_u(P, V, U, L, rows, st, s, df));
     CHECK(precondition_into(c, U, Gk, T, L, j, mode, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op), launch_apply_f64(op, Gk, Y, L, s));
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, Gk, Y, field, L, s));
     LAUNCH(WD_K_UPDATE_XR, 2, launch_update_xr(jp.X, F, Gk, R, W, Y, Rt, L, rows, part, st, s, df));
     graph_iter_check<<<1, 32, 0, s>>>(st, g, hist, hloop, htail);
     CU(cudaGetLastError());
@@ -1467,7 +1522,7 @@ int build_run(wd_ctx* c, const JobPtrs& jp, int mode, bool df, bool restore, cud
   cudaGraph_t tail = ip.conditional.phGraph_out[0];
   CHECK(capture_into(c, tail, {}, [&](cudaStream_t s) -> int {
     CHECK(precondition_into(c, R, F, T, L, j, mode, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op), launch_apply_f64(op, F, W, L, s));
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, F, W, field, L, s));
     LAUNCH(WD_K_TRACE, 2, launch_traces(W, R, L, rows, part, st, s));
     LAUNCH(WD_K_SOLVE_LL, 1, launch_solve_gamma(st, L, s));
     LAUNCH(WD_K_UPDATE_PV, 2, launch_update_pv(P, V, R, W, U, Y, Rt, L, rows, part, st, s, df));
@@ -1499,6 +1554,7 @@ int build_job(wd_ctx* c, const JobPtrs& jp, cudaGraph_t G) {
   double2* part = static_cast<double2*>(c->part.p);
   GraphCtl* g = static_cast<GraphCtl*>(c->gctl);
   const bool two_modes = jp.X0 != nullptr;
+  void* const field = op.apply_form == 1 ? c->field.p : nullptr;
 
   cudaGraphConditionalHandle hphase;
   CU(cudaGraphConditionalHandleCreate(&hphase, G, 1, cudaGraphCondAssignDefault));
@@ -1528,7 +1584,7 @@ int build_job(wd_ctx* c, const JobPtrs& jp, cudaGraph_t G) {
   }
   // the true residual of the pass, then the decision
   CHECK(capture_into(c, pass, {two_modes ? nrun1 : nrun0}, [&](cudaStream_t s) -> int {
-    LAUNCH(WD_K_RESID, stencil_kernels(op), launch_resid_f64(op, jp.X, jp.B, T, L, s));
+    LAUNCH(WD_K_RESID, stencil_kernels(op, field), launch_resid_f64(op, jp.X, jp.B, T, field, L, s));
     LAUNCH(WD_K_COLNORM, 2, launch_colnorms(T, L, rows, part, g->true2, s));
     graph_phase_end<<<1, 32, 0, s>>>(g, hphase);
     CU(cudaGetLastError());
@@ -1568,6 +1624,7 @@ extern "C" int bbicggr_solve_batch(bbicggr_job* jobs, int njobs, void* stream) {
     bbicggr_job& jb = jobs[i];
     wd_ctx* c = jb.ctx;
     CHECK(ensure_workspace(c, jb.L));
+    field_block(c, jb.L, s);
     const int mode = precond_mode(jb.opts);
     if ((mode == PM_F32 || mode == PM_BF16) && jb.j >= 2)
       CHECK(ensure_workspace_lp(c, lp_storage(mode), jb.L, s));

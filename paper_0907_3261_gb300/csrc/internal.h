@@ -34,35 +34,54 @@ struct Op {
   // [site][chirality][36 floats] (the packed blocks of clov_inv32).
   float4* links32s;
   float4* clov_inv32s;
-  // The FP32-lane form of the FP64 stencil (dslash_x3.cu): the links cut into three FP32 levels,
-  // [site][mu][level][entry] as (re, re, im, im) (null when the links are not unitary), a scratch
-  // of V * WD_LMAX exponents, and the form in use (1: this one, 0: the FP64-pipe kernel).
-  float4* links_x3;
-  int* xexp;
+  // The fixed-point form of the FP64 stencil (dslash_fx.cu; null tables when the links are not
+  // unitary): kappa times the eight links of every site [site][direction][row][column], A_D and
+  // A_D^{-1} [site][chirality][row][column] with their exponents, every entry a complex integer in
+  // limbs; the eight neighbours of every site; the links' scale; three sets of V * WD_LMAX exponents
+  // (two for ping-ponged fields, one for the sweeps' right-hand side); and the form in use (1: this
+  // one, 0: the FP64-pipe kernel).
+  int4* fx_links;
+  int4* fx_clov;
+  int4* fx_cinv;
+  int4* fx_nb;
+  short* fx_exps;
+  int fx_ek;
   int apply_form;
+  short* fx_exp(int slot) const { return fx_exps + (size_t)slot * g.V * WD_LMAX; }
 };
+constexpr int FX_WSTR = 72;   // int4 per site of fx_links
+constexpr int FX_DSTR = 73;   // int4 per site of fx_clov, fx_cinv
 
 // Largest entry error |row2 - conj(row0 x row1)| of a link that still counts as special unitary.
 constexpr double LINK12_TOL = 1e-6;
 
-// ---- dslash.cu (FP64)
-cudaError_t launch_apply_f64(const Op& op, const double* x, double* y, int L, cudaStream_t st);
-cudaError_t launch_resid_f64(const Op& op, const double* x, const double* b, double* y, int L,
+// ---- dslash.cu (FP64).  `field` is a block for the fixed-point form's copy of x; without one, or
+// with apply_form 0, the product runs on the FP64 pipe.
+cudaError_t launch_apply_f64(const Op& op, const double* x, double* y, void* field, int L,
                              cudaStream_t st);
+cudaError_t launch_resid_f64(const Op& op, const double* x, const double* b, double* y, void* field,
+                             int L, cudaStream_t st);
+// One FP64-pipe Jacobi sweep, and the first one from G = 0.
 cudaError_t launch_jacobi_f64(const Op& op, const double* g_in, const double* u, double* g_out,
                               int L, cudaStream_t st);
 cudaError_t launch_site_inverse_f64(const Op& op, const double* u, double* g_out, int L,
                                     cudaStream_t st);
 
-// ---- dslash_x3.cu (the same FP64 operations with the hopping sums on the FP32 lanes)
-cudaError_t launch_link_split(const Op& op, cudaStream_t st);
-cudaError_t launch_apply_x3(const Op& op, const double* x, double* y, int L, cudaStream_t st);
-cudaError_t launch_resid_x3(const Op& op, const double* x, const double* b, double* y, int L,
+// ---- dslash_fx.cu (the same FP64 operations in 64-bit fixed point)
+int fx_link_exponent(double kappa);
+cudaError_t launch_fx_tables(const Op& op, cudaStream_t st);
+cudaError_t launch_apply_fx(const Op& op, const double* x, double* y, void* field, int L,
                             cudaStream_t st);
-cudaError_t launch_jacobi_x3(const Op& op, const double* g_in, const double* u, double* g_out,
-                             int L, cudaStream_t st);
-// Kernels one FP64 stencil launch takes (the x3 form adds its exponent pre-pass).
-inline int stencil_kernels(const Op& op) { return op.apply_form == 1 ? 2 : 1; }
+cudaError_t launch_resid_fx(const Op& op, const double* x, const double* b, double* y, void* field,
+                            int L, cudaStream_t st);
+// The sweeps' iterates are fields (as large as FP64 blocks) with their exponents in slot 0 or 1.  The
+// first sweep from G = 0 also records u's exponents, which the later ones read; a sweep writes a field
+// with its exponents in the other slot (q_out), or FP64 (g64).
+cudaError_t launch_first_fx(const Op& op, const double* u, void* q_out, int slot, int L, cudaStream_t st);
+cudaError_t launch_sweep_fx(const Op& op, const void* q_in, int slot, const double* u, void* q_out,
+                            double* g64, int L, cudaStream_t st);
+// Kernels one FP64 product with A takes (the fixed-point form copies its operand first).
+inline int stencil_kernels(const Op& op, const void* field) { return op.apply_form == 1 && field ? 2 : 1; }
 
 // ---- sweep_lp.cu, sweep_f32.cu, sweep_bf16.cu: the low-precision preconditioner.  Its private
 // blocks (u_lp, g_lp) are component-major, [spin*3+colour][site][rhs], one complex number per
