@@ -1,0 +1,712 @@
+// The products of the block recurrences (arXiv:0907.3261, Sec. 2, the algorithm box) on the tensor cores in
+// exact digits: block times L x L matrix (U = S alpha, P = R + U gamma, V = W + Y gamma) and the L x L Gram
+// products R~_0^H R and R~_0^H V, fused with the updates that feed them.
+//
+// GB300's FP64 pipe issues two lanes per clock per SM, and a complex multiply-add in FP32 pairs takes about 20
+// packed instructions, so these products bounded the updates.  Here every factor is an integer of ND
+// balanced base-256 digits (ND = 7: 55 bits and the sign, ND = 8: 63), and a digit is an FP16 number: the
+// products of digits and their sums, below 2^22, are exact in mma.sync's FP32 accumulators.  One accumulator
+// per order (the sum of the two digits' positions) for the orders 0 .. ND - 1, started at 1.5 2^23, whose
+// bits are then the sum as an integer; what is dropped is below 2^-8ND of the largest product.  mma.sync and
+// not tcgen05: a tile is 16 rows by at most 32 columns, and the thread that loads an element also
+// owns the element of the same place in the product, so nothing but the digits of alpha and gamma passes
+// through shared memory.
+//
+// Scales: in block times matrix, a power of two per row of the block, per row and per column of the
+// matrix (its entries are first divided by their row's scale, which goes to the block's column, so a block
+// with columns of very different size loses nothing).  In a Gram product, a power of two per column of
+// either block, held by a warp from tile to tile while the columns' largest elements stay within 2^-7 of
+// it; the warp's sums are 64-bit integers and go to FP64 when a scale changes or after GR_TILES tiles.
+// An infinity or a NaN makes its row of a product, and its row or column of a Gram product, NaN.
+//
+// A warp takes 16 rows at a time: thread (g, t) = (lane / 4, lane % 4) holds rows g, g + 8 and columns
+// t + 4 i, i < NI = ceil(L / 4).  That is the layout of an mma A fragment with (re, im) as its pairs, and of
+// the accumulators, so products need no exchange; a Gram product contracts over the rows, and movmatrix
+// transposes the digits of both blocks.  Partial sums are added in a fixed order, bitwise reproducible.
+//
+// Measured on a GB300, 16^3x32, L = 12, with the call's 50 us: U 0.29 ms against 0.62 in FP32 pairs and 1.76
+// on the FP64 pipe; P and V 0.98 against 1.81 and 4.90; X and R 0.69 against 0.95 and 2.66.  L = 1: 0.10,
+// 0.26 and 0.26 ms against 0.10, 0.36 and 0.46 (FP32 pairs); 4^4, L = 4: as before, 35 to 60 us.  Bytes alone
+// would take 0.14, 0.32 and 0.41 ms.  X and R is at 76% of the FP64 pipe (their updates stay FP64); the others
+// are bound by the latency of a tile's chain at 12 to 16 warps per SM (tensor pipe 33 to 44%, integer pipe
+// 35 to 42%).  P and V in three blocks of 168 registers against four of 128 and spills: 0.98 against 1.01 ms
+// (L = 16: 1.38 against 1.57); two copies of the product's code for U and Y, 1.08.  Scales without a bit to
+// spare, more flushes: 1.15 ms.
+#include <type_traits>
+
+#include "fixed.cuh"
+#include "internal.h"
+
+namespace {
+
+using fx::i64;
+using fx::u64;
+
+constexpr int DG_TPB = 128;                // 4 warps
+constexpr int DG_WARPS = DG_TPB / 32;
+constexpr int GR_TILES = 8;                // |tile sum| <= 2^59.1: 8 of them stay below 2^63
+constexpr int GR_WINDOW = 7;               // bits by which a column may fall below its scale
+constexpr int DG_BAD = 1 << 20;            // an exponent that marks an infinity or a NaN
+constexpr unsigned DG_MAGIC = 0x4B400000u;   // 1.5 2^23
+
+WD_DEV void mma16(float c[4], const unsigned a[4], unsigned b0, unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+WD_DEV void mma8(float c[4], unsigned a0, unsigned a1, unsigned b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5},{%6},{%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(b0));
+}
+WD_DEV unsigned transposed(unsigned a) {
+  unsigned d;
+  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(d) : "r"(a));
+  return d;
+}
+WD_DEV unsigned hfma2(unsigned a, unsigned b, unsigned c) {
+  unsigned d;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;\n" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+WD_DEV int raw_exponent(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
+
+// |v| >> sh as an integer of 8 ND - 1 bits for a v in [1, 2) 2^e at sh = 0, plus 128 in every byte below the
+// top digit's.  FP64 subnormals count as zero.
+template <int ND>
+WD_DEV u64 biased(double v, int e_minus_scale) {
+  const int h = __double2hiint(v);
+  const int sh = (h & 0x7FF00000) ? -e_minus_scale : 64;
+  const u64 m = ((u64)(unsigned)((h & 0xFFFFF) | 0x100000) << 32 | (unsigned)__double2loint(v))
+                << (ND == 8 ? 10 : 2);
+  return fx::shr_u(m, sh) + (ND == 8 ? 0x0080808080808080ull : 0x0000808080808080ull);
+}
+// v as a digit integer for the scale E: |v| < 2^(E - 1022), e added to v's exponent.
+template <int ND>
+WD_DEV u64 biased_at(double v, int e, int E) {
+  return biased<ND>(v, raw_exponent(v) + e - E);
+}
+// The ND digits of x and y (biased magnitudes, signs from the words hx, hy) as FP16 pairs, most significant
+// first: the bytes b become 1024 + b, and (1024 + b) s - 1152 s is the digit (the top one has no bias).
+template <int ND>
+WD_DEV void digits(u64 x, u64 y, int hx, int hy, unsigned d[ND]) {
+  const unsigned p = __byte_perm(hx, hy, 0x7030) & 0x80008000u;
+  const unsigned s = p | 0x3C003C00u, c = p ^ 0xE480E480u, ct = p ^ 0xE400E400u;
+  const unsigned xl = (unsigned)x, yl = (unsigned)y, xh = (unsigned)(x >> 32), yh = (unsigned)(y >> 32);
+  const unsigned w[4] = {__byte_perm(xl, yl, 0x5140), __byte_perm(xl, yl, 0x7362),
+                         __byte_perm(xh, yh, 0x5140), __byte_perm(xh, yh, 0x7362)};
+#pragma unroll
+  for (int j = 0; j < ND; ++j)
+    d[ND - 1 - j] = hfma2(__byte_perm(w[j >> 1], 0x64646464u, (j & 1) ? 0x4342 : 0x4140), s,
+                          j == ND - 1 ? ct : c);
+}
+
+// v 2^k, rounded once.  The FP64 pipe's conversions would take 130 cycles of it per warp.
+WD_DEV double scaled(i64 v, int k) {
+  const i64 sg = v >> 63;
+  const u64 m = (u64)((v ^ sg) - sg);
+  const int n = __clzll((i64)m);
+  const u64 q = (((m << (n & 63)) >> 10) + 1) >> 1;
+  const int h = (int)(q >> 32) + ((1085 - n + k) << 20);
+  return m ? __hiloint2double(h | ((int)(sg) & 0x80000000), (int)q) : 0.0;
+}
+__device__ __noinline__ double scaled_any(i64 v, int k) { return ldexp(scaled(v, 0), k); }
+WD_DEV double2 scaled2(i64 re, i64 im, int k) {
+  if ((unsigned)(k + 1000) < 1900u) return make_double2(scaled(re, k), scaled(im, k));
+  if (k < DG_BAD / 2) return make_double2(scaled_any(re, k), scaled_any(im, k));
+  const double nan = __longlong_as_double(0x7FF8000000000000LL);
+  return make_double2(nan, nan);
+}
+
+// Sums of the orders as an integer (j: accumulator bits, b: the bits that stand for zero), the order 0 in
+// units of 2^(40 + UP); the orders 6 and 7 are rounded (a floor's bias would grow with the rows of a Gram
+// product).
+template <int ND, int UP>
+WD_DEV i64 joined(const int j[ND], unsigned b) {
+  const int A = (int)((unsigned)(j[0] << 8) + j[1] - 257u * b), B = (int)((unsigned)(j[2] << 8) + j[3] - 257u * b);
+  const int C = (int)((unsigned)(j[4] << 8) + j[5] - 257u * b);
+  int D;
+  if constexpr (ND == 8) D = (int)((unsigned)(j[6] << 8) + j[7] - 257u * b + (1u << (15 - UP))) >> (16 - UP);
+  else D = (int)(j[6] - b + (1u << (7 - UP))) >> (8 - UP);
+  return (i64)B * (1 << (16 + UP)) + ((i64)C * (1 << UP) + D) + ((i64)A << (32 + UP));
+}
+
+// ---------------------------------------------------------------- block times matrix
+// The digits of an L x L matrix as mma B fragments, and its scales.
+template <int NI, int ND>
+struct Coef {
+  unsigned d[NI * NI * ND * 32];           // [column tile][entry group][digit][lane]
+  int row[4 * NI], col[4 * NI];            // exponents: |m_ab| < 2^(row + col - 1022)
+};
+
+// Fills `t` from the matrix m, staged in `st` (L^2 entries); ends with a barrier.
+template <int NI, int ND>
+WD_DEV void load_coef(Coef<NI, ND>& t, double2* st, const double2* __restrict__ m, int L) {
+  const int tid = threadIdx.x;
+  if (tid < 4 * NI) t.row[tid] = t.col[tid] = 0;
+  __syncthreads();
+  // exponent fields: 0 for zero, 2047 for an infinity or a NaN, which do not count for a row's scale
+  for (int e = tid; e < L * L; e += DG_TPB) {
+    const double2 v = st[e] = m[e];
+    const int x = fx::exponent_of(v);
+    if (x && x < 2047) atomicMax(&t.row[e / L], x);
+  }
+  __syncthreads();
+  if (tid < 4 * NI) t.row[tid] = t.row[tid] ? t.row[tid] - 1023 : 0;
+  __syncthreads();
+  // columns, shifted by 4096 so that zero stands for none
+  for (int e = tid; e < L * L; e += DG_TPB) {
+    const int x = fx::exponent_of(st[e]), a = e / L;
+    if (x) atomicMax(&t.col[e - a * L], x == 2047 ? DG_BAD : 4096 + x - t.row[a]);
+  }
+  __syncthreads();
+  if (tid < 4 * NI) t.col[tid] = t.col[tid] == 0 ? 1023 : t.col[tid] == DG_BAD ? DG_BAD : t.col[tid] - 4096;
+  __syncthreads();
+  for (int q = tid; q < NI * NI * 32; q += DG_TPB) {
+    const int lane = q & 31, ni = q >> 5, i = ni % NI, nt = ni / NI;
+    const int a = (lane & 3) + 4 * i, b = (lane >> 3) + 4 * nt;
+    double2 v = make_double2(0.0, 0.0);
+    if (a < L && b < L) v = st[a * L + b];
+    // column 2b of the real matrix has (re, -im) in rows 2a, 2a + 1, column 2b + 1 (im, re)
+    const double x = (lane & 4) ? v.y : v.x, y = (lane & 4) ? v.x : -v.y;
+    unsigned d[ND];
+    digits<ND>(biased_at<ND>(x, -t.row[a], t.col[b]), biased_at<ND>(y, -t.row[a], t.col[b]),
+               __double2hiint(x), __double2hiint(y), d);
+#pragma unroll
+    for (int k = 0; k < ND; ++k) t.d[(ni * ND + k) * 32 + lane] = d[k];
+  }
+  __syncthreads();
+}
+
+// The product of the warp's 16 rows with the matrix: put(h, nt, v) gets element (row g + 8 h, column
+// t + 4 nt).
+template <int NI, int ND, class G, class F>
+WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, const G& get, const F& put) {
+  const int lane = threadIdx.x & 31;
+  unsigned a[ND][2][NI];
+  int E[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int ra[NI];
+    E[h] = -4000;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      ra[i] = t.row[(lane & 3) + 4 * i];
+      const int e = fx::exponent_of(in[h][i]);
+      E[h] = max(E[h], e == 2047 ? DG_BAD : e ? e + ra[i] : -4000);
+    }
+    E[h] = max(E[h], __shfl_xor_sync(0xFFFFFFFFu, E[h], 1));
+    E[h] = max(E[h], __shfl_xor_sync(0xFFFFFFFFu, E[h], 2));
+    if (E[h] == -4000) E[h] = 1023;        // a row of zeros
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const double2 v = in[h][i];
+      unsigned d[ND];
+      digits<ND>(biased_at<ND>(v.x, ra[i], E[h]), biased_at<ND>(v.y, ra[i], E[h]), __double2hiint(v.x),
+                 __double2hiint(v.y), d);
+#pragma unroll
+      for (int k = 0; k < ND; ++k) a[k][h][i] = d[k];
+    }
+  }
+#pragma unroll 1
+  for (int nt = 0; nt < NI; ++nt) {
+    const double2 base[2] = {get(0, nt), get(1, nt)};
+    float acc[ND][4];
+#pragma unroll
+    for (int o = 0; o < ND; ++o)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[o][q] = __uint_as_float(DG_MAGIC);
+    const unsigned* bd = t.d + nt * NI * ND * 32 + lane;
+#pragma unroll
+    for (int i = 0; i + 1 < NI; i += 2) {
+#pragma unroll
+      for (int k2 = 0; k2 < ND; ++k2) {
+        const unsigned b0 = bd[(i * ND + k2) * 32], b1 = bd[((i + 1) * ND + k2) * 32];
+#pragma unroll
+        for (int k1 = 0; k1 + k2 < ND; ++k1) {
+          const unsigned f[4] = {a[k1][0][i], a[k1][1][i], a[k1][0][i + 1], a[k1][1][i + 1]};
+          mma16(acc[k1 + k2], f, b0, b1);
+        }
+      }
+    }
+    if constexpr (NI & 1) {
+#pragma unroll
+      for (int k2 = 0; k2 < ND; ++k2) {
+        const unsigned b0 = bd[((NI - 1) * ND + k2) * 32];
+#pragma unroll
+        for (int k1 = 0; k1 + k2 < ND; ++k1)
+          mma8(acc[k1 + k2], a[k1][0][NI - 1], a[k1][1][NI - 1], b0);
+      }
+    }
+    const int C = t.col[(lane & 3) + 4 * nt];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int re[ND], im[ND];
+#pragma unroll
+      for (int o = 0; o < ND; ++o) {
+        re[o] = __float_as_int(acc[o][2 * h]);
+        im[o] = __float_as_int(acc[o][2 * h + 1]);
+      }
+      put(h, nt, base[h], scaled2(joined<ND, 3>(re, DG_MAGIC), joined<ND, 3>(im, DG_MAGIC), E[h] + C - 2101));
+    }
+  }
+}
+
+// ---------------------------------------------------------------- Gram product
+// One warp's A^H B: element (a, b), a = 8 mt + 4 (g % 2) + g / 2 and b = t + 4 nt, belongs to thread (g, t).
+template <int NI, int ND>
+struct Gram {
+  static constexpr int MT = (NI + 1) / 2, NV = MT * NI * 2, LD = 4 * NI;
+  i64* sum;                                // [NV][DG_TPB], this thread's slots
+  double2* out;                            // [LD][LD] of this warp
+  int ea[NI], eb[NI], tiles;
+  unsigned bad;                            // bits i: column t + 4 i of A, 8 + i: of B holds an infinity or a NaN
+
+  WD_DEV void init(i64* s, double2* o) {
+    sum = s;
+    out = o;
+    tiles = 0;
+    bad = 0;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) ea[i] = eb[i] = -1;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) sum[q * DG_TPB] = 0;
+    for (int e = threadIdx.x & 31; e < LD * LD; e += 32) out[e] = make_double2(0.0, 0.0);
+    __syncwarp();
+  }
+  WD_DEV void flush() {
+    const int lane = threadIdx.x & 31, g = lane >> 2, tt = lane & 3;
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+      const int e0 = __shfl_sync(0xFFFFFFFFu, ea[2 * mt], g >> 1);
+      const int e1 = 2 * mt + 1 < NI ? __shfl_sync(0xFFFFFFFFu, ea[2 * mt + 1 < NI ? 2 * mt + 1 : 0], g >> 1) : 0;
+      const int E = (g & 1) ? e1 : e0, a = 8 * mt + 4 * (g & 1) + (g >> 1);
+#pragma unroll
+      for (int nt = 0; nt < NI; ++nt) {
+        i64* s = sum + (mt * NI + nt) * 2 * DG_TPB;
+        const double2 v = scaled2(s[0], s[DG_TPB], E + eb[nt] - 2098);
+        if (a < LD) {
+          double2& o = out[a * LD + tt + 4 * nt];
+          o = make_double2(o.x + v.x, o.y + v.y);
+        }
+        s[0] = 0;
+        s[DG_TPB] = 0;
+      }
+    }
+    tiles = 0;
+  }
+  // Scales for the columns of a tile; true when some column left its window.
+  WD_DEV static int column(const double2 v[2][NI], int i, unsigned& bad, int bit) {
+    int e = max(fx::exponent_of(v[0][i]), fx::exponent_of(v[1][i]));
+    if (e == 2047) {
+      bad |= 1u << bit;
+      e = 2046;
+    }
+    e = max(e, __shfl_xor_sync(0xFFFFFFFFu, e, 4));
+    e = max(e, __shfl_xor_sync(0xFFFFFFFFu, e, 8));
+    return max(e, __shfl_xor_sync(0xFFFFFFFFu, e, 16));
+  }
+  WD_DEV void tile(const double2 A[2][NI], const double2 B[2][NI]) {
+    {
+      int na[NI], nb[NI];
+      bool moved = tiles == GR_TILES;
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        na[i] = column(A, i, bad, i);
+        nb[i] = column(B, i, bad, 8 + i);
+        moved = moved || na[i] > ea[i] || nb[i] > eb[i] || (na[i] && na[i] < ea[i] - GR_WINDOW) ||
+                (nb[i] && nb[i] < eb[i] - GR_WINDOW);
+      }
+      if (__any_sync(0xFFFFFFFFu, moved)) {
+        if (tiles) flush();
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          if (na[i] || ea[i] < 0) ea[i] = na[i] + (ea[i] >= 0);   // from the second time on with a bit to spare
+          if (nb[i] || eb[i] < 0) eb[i] = nb[i] + (eb[i] >= 0);
+        }
+      }
+      ++tiles;
+    }
+    unsigned b[NI][2][ND];
+#pragma unroll
+    for (int nt = 0; nt < NI; ++nt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const double2 v = B[h][nt];
+        digits<ND>(biased_at<ND>(v.x, 0, eb[nt]), biased_at<ND>(v.y, 0, eb[nt]), __double2hiint(v.x),
+                   __double2hiint(v.y), b[nt][h]);
+#pragma unroll
+        for (int k = 0; k < ND; ++k) b[nt][h][k] = transposed(b[nt][h][k]);
+      }
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+      unsigned a[ND][4];                   // rows g: real parts, rows g + 8: imaginary parts
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        double2 v[2];
+        int e[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {      // columns 2 mt + c
+          const bool lo = MT == 1 || mt == 0;
+          v[c] = lo ? (c < NI ? A[h][c < NI ? c : 0] : make_double2(0.0, 0.0))
+                    : (2 + c < NI ? A[h][2 + c < NI ? 2 + c : 0] : make_double2(0.0, 0.0));
+          e[c] = lo ? ea[c < NI ? c : 0] : ea[2 + c < NI ? 2 + c : 0];
+        }
+        unsigned d[ND];
+        digits<ND>(biased_at<ND>(v[0].x, 0, e[0]), biased_at<ND>(v[1].x, 0, e[1]), __double2hiint(v[0].x),
+                   __double2hiint(v[1].x), d);
+#pragma unroll
+        for (int k = 0; k < ND; ++k) a[k][2 * h] = transposed(d[k]);
+        digits<ND>(biased_at<ND>(v[0].y, 0, e[0]), biased_at<ND>(v[1].y, 0, e[1]), __double2hiint(v[0].y),
+                   __double2hiint(v[1].y), d);
+#pragma unroll
+        for (int k = 0; k < ND; ++k) a[k][2 * h + 1] = transposed(d[k]);
+      }
+#pragma unroll
+      for (int nt = 0; nt < NI; ++nt) {
+        float acc[ND][4];
+#pragma unroll
+        for (int o = 0; o < ND; ++o)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[o][q] = __uint_as_float(DG_MAGIC);
+#pragma unroll
+        for (int k2 = 0; k2 < ND; ++k2)
+#pragma unroll
+          for (int k1 = 0; k1 + k2 < ND; ++k1) mma16(acc[k1 + k2], a[k1], b[nt][0][k2], b[nt][1][k2]);
+        int re[ND], im[ND];
+#pragma unroll
+        for (int o = 0; o < ND; ++o) {
+          re[o] = __float_as_int(acc[o][0]) + __float_as_int(acc[o][3]);
+          im[o] = __float_as_int(acc[o][1]) - __float_as_int(acc[o][2]);
+        }
+        i64* s = sum + (mt * NI + nt) * 2 * DG_TPB;
+        s[0] += joined<ND, 0>(re, 2u * DG_MAGIC);
+        s[DG_TPB] += joined<ND, 0>(im, 0u);
+      }
+    }
+  }
+  // The block's sums into its slot of the partial sums; `nacc`: this thread's column norms, or null.
+  WD_DEV void write(double2* __restrict__ part, const double2* all, double* nred, int L, const double* nacc) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    flush();
+    unsigned m = bad;
+#pragma unroll
+    for (int k = 4; k < 32; k <<= 1) m |= __shfl_xor_sync(0xFFFFFFFFu, m, k);
+    const double nan = __longlong_as_double(0x7FF8000000000000LL);
+    __syncwarp();
+    if (lane < 4) {
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+        for (int q = 0; q < LD; ++q) {
+          if (m >> i & 1) out[(lane + 4 * i) * LD + q] = make_double2(nan, nan);
+          if (m >> (8 + i) & 1) out[q * LD + lane + 4 * i] = make_double2(nan, nan);
+        }
+    }
+    if (nacc) {
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        double v = nacc[i];
+#pragma unroll
+        for (int k = 4; k < 32; k <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, k);
+        if (lane < 4) nred[w * 16 + lane + 4 * i] = v;
+      }
+    }
+    __syncthreads();
+    double2* p = part + (size_t)blockIdx.x * PART_STRIDE;
+    for (int e = threadIdx.x; e < L * L; e += DG_TPB) {
+      const int a = e / L, b = e - a * L;
+      double2 v = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int k = 0; k < DG_WARPS; ++k) {
+        const double2 x = all[k * LD * LD + a * LD + b];
+        v.x += x.x;
+        v.y += x.y;
+      }
+      p[e] = v;
+    }
+    if (nacc && threadIdx.x < L) {
+      double v = 0.0;
+#pragma unroll
+      for (int k = 0; k < DG_WARPS; ++k) v += nred[k * 16 + threadIdx.x];
+      p[WD_LMAX * WD_LMAX + threadIdx.x] = make_double2(v, 0.0);
+    }
+  }
+};
+
+// This thread's elements of a tile's rows; `e` and `ok` from Place.
+template <int NI>
+struct Place {
+  size_t e[2];                             // element (row g + 8 h, column t)
+  bool row[2];
+  int left;                                // columns left from t on
+  WD_DEV Place(long long tile, int L, long long rows) {
+    const int lane = threadIdx.x & 31;
+    left = L - (lane & 3);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const long long n = tile * 16 + (lane >> 2) + 8 * h;
+      row[h] = n < rows;
+      e[h] = (size_t)n * L + (lane & 3);
+    }
+  }
+  WD_DEV bool ok(int h, int i) const { return row[h] && 4 * i < left; }
+  WD_DEV void load(const double* __restrict__ p, double2 v[2][NI]) const {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+        v[h][i] = ok(h, i) ? reinterpret_cast<const double2*>(p)[e[h] + 4 * i] : make_double2(0.0, 0.0);
+  }
+};
+// A tile's elements on their way to the thread that asked for them: its own slots of shared memory, so a
+// wait of the thread is all that a read needs.
+template <int NI>
+struct Staged {
+  double2 slot[2 * NI][DG_TPB];
+  WD_DEV void ask(const Place<NI>& pl, const double* __restrict__ p) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const bool ok = pl.ok(h, i);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(&slot[h * NI + i][threadIdx.x])),
+                     "l"(ok ? p + 2 * (pl.e[h] + 4 * i) : p), "r"(ok ? 16 : 0)
+                     : "memory");
+      }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+  WD_DEV void take(double2 v[2][NI]) {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < NI; ++i) v[h][i] = slot[h * NI + i][threadIdx.x];
+  }
+};
+WD_DEV double2& at(double* p, size_t e) { return reinterpret_cast<double2*>(p)[e]; }
+WD_DEV double2 at(const double* p, size_t e) { return reinterpret_cast<const double2*>(p)[e]; }
+// t + z f
+WD_DEV double2 axpy(double2 t, double2 z, double2 f) {
+  return make_double2(fma(-z.y, f.y, fma(z.x, f.x, t.x)), fma(z.y, f.x, fma(z.x, f.y, t.y)));
+}
+
+// U = (P - zeta V) alpha
+template <int NI, int ND>
+__global__ void __launch_bounds__(DG_TPB, 4)
+update_u_dg_kernel(const double* __restrict__ P, const double* __restrict__ V, double* __restrict__ U, int L,
+                   long long rows, const SolverState* __restrict__ st) {
+  __shared__ Coef<NI, ND> al;
+  __shared__ Staged<NI> sp, sv;            // sp is also the matrix's stage
+  if (st->status != ST_OK) return;
+  const double2 z = st->zeta, mz = make_double2(-z.x, -z.y);
+  load_coef(al, &sp.slot[0][0], st->alpha, L);
+  const long long tiles = (rows + 15) / 16, step = (long long)gridDim.x * DG_WARPS;
+  long long q = (long long)blockIdx.x * DG_WARPS + (threadIdx.x >> 5);
+  if (q < tiles) {
+    const Place<NI> pl(q, L, rows);
+    sp.ask(pl, P);
+    sv.ask(pl, V);
+  }
+  for (; q < tiles; q += step) {
+    const Place<NI> pl(q, L, rows);
+    double2 s[2][NI], v[2][NI];
+    sp.take(s);
+    sv.take(v);
+    if (q + step < tiles) {
+      const Place<NI> next(q + step, L, rows);
+      sp.ask(next, P);
+      sv.ask(next, V);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < NI; ++i) s[h][i] = axpy(s[h][i], mz, v[h][i]);
+    row_product<NI, ND>(
+        s, al, [](int, int) { return make_double2(0.0, 0.0); },
+        [&](int h, int nt, double2, double2 u) {
+          if (pl.ok(h, nt)) at(U, pl.e[h] + 4 * nt) = u;
+        });
+  }
+}
+
+// Partial A^H B, and the column norms of B.
+template <int NI, int ND>
+__global__ void __launch_bounds__(DG_TPB, NI == 4 ? 3 : 4)
+gram_dg_kernel(const double* __restrict__ A, const double* __restrict__ B, int L, long long rows,
+               double2* __restrict__ part, bool norms) {
+  using Gr = Gram<NI, ND>;
+  __shared__ i64 sums[Gr::NV][DG_TPB];
+  __shared__ double2 outs[DG_WARPS][Gr::LD * Gr::LD];
+  __shared__ double nred[DG_WARPS * 16];
+  Gr gr;
+  gr.init(&sums[0][threadIdx.x], outs[threadIdx.x >> 5]);
+  double nacc[NI] = {};
+  const long long tiles = (rows + 15) / 16;
+  for (long long q = (long long)blockIdx.x * DG_WARPS + (threadIdx.x >> 5); q < tiles;
+       q += (long long)gridDim.x * DG_WARPS) {
+    const Place<NI> pl(q, L, rows);
+    double2 a[2][NI], b[2][NI];
+    pl.load(A, a);
+    pl.load(B, b);
+    if (norms) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < NI; ++i) nacc[i] = fma(b[h][i].x, b[h][i].x, fma(b[h][i].y, b[h][i].y, nacc[i]));
+    }
+    gr.tile(a, b);
+  }
+  gr.write(part, outs[0], nred, L, norms ? nacc : nullptr);
+}
+
+// X += zeta F + G;  R -= zeta W + Y;  partial R~_0^H R_{k+1} and ||r_i||^2.
+template <int NI, int ND>
+__global__ void __launch_bounds__(DG_TPB, NI == 4 ? 3 : 4)
+update_xr_dg_kernel(double* __restrict__ X, const double* __restrict__ F, const double* __restrict__ G,
+                    double* __restrict__ R, const double* __restrict__ W, const double* __restrict__ Y,
+                    const double* __restrict__ Rt, int L, long long rows, double2* __restrict__ part,
+                    const SolverState* __restrict__ st) {
+  using Gr = Gram<NI, ND>;
+  __shared__ __align__(16) i64 sums[Gr::NV][DG_TPB];
+  __shared__ double2 outs[DG_WARPS][Gr::LD * Gr::LD];
+  __shared__ double nred[DG_WARPS * 16];
+  if (st->status != ST_OK) return;
+  const double2 z = st->zeta, mz = make_double2(-z.x, -z.y);
+  Gr gr;
+  gr.init(&sums[0][threadIdx.x], outs[threadIdx.x >> 5]);
+  double nacc[NI] = {};
+  const long long tiles = (rows + 15) / 16;
+  for (long long q = (long long)blockIdx.x * DG_WARPS + (threadIdx.x >> 5); q < tiles;
+       q += (long long)gridDim.x * DG_WARPS) {
+    const Place<NI> pl(q, L, rows);
+    double2 r[2][NI], rt[2][NI];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const size_t e = pl.e[h] + 4 * i;
+        r[h][i] = make_double2(0.0, 0.0);
+        if (!pl.ok(h, i)) continue;
+        const double2 x = at(X, e), g = at(G, e), y = at(Y, e);
+        r[h][i] = at(R, e);
+        at(X, e) = axpy(make_double2(x.x + g.x, x.y + g.y), z, at(F, e));
+        r[h][i] = axpy(make_double2(r[h][i].x - y.x, r[h][i].y - y.y), mz, at(W, e));
+        at(R, e) = r[h][i];
+        nacc[i] = fma(r[h][i].x, r[h][i].x, fma(r[h][i].y, r[h][i].y, nacc[i]));
+      }
+    pl.load(Rt, rt);
+    gr.tile(rt, r);
+  }
+  gr.write(part, outs[0], nred, L, nacc);
+}
+
+// P = R + U gamma;  V = W + Y gamma;  partial R~_0^H V_{k+1}.
+template <int NI, int ND>
+__global__ void __launch_bounds__(DG_TPB, NI >= 3 ? 3 : 4)
+update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double* __restrict__ R,
+                    const double* __restrict__ W, const double* __restrict__ U, const double* __restrict__ Y,
+                    const double* __restrict__ Rt, int L, long long rows, double2* __restrict__ part,
+                    const SolverState* __restrict__ st) {
+  using Gr = Gram<NI, ND>;
+  __shared__ Coef<NI, ND> ga;
+  __shared__ __align__(16) i64 sums[Gr::NV][DG_TPB];
+  __shared__ double2 outs[DG_WARPS][Gr::LD * Gr::LD];
+  constexpr bool ST = NI < 4;              // NI = 4: beyond 48 KB of static shared memory
+  __shared__ Staged<ST ? NI : 1> sg_;
+  Staged<NI>& sg = reinterpret_cast<Staged<NI>&>(sg_);
+  if (st->status != ST_OK) return;
+  const long long tiles = (rows + 15) / 16, step = (long long)gridDim.x * DG_WARPS;
+  const long long q0 = (long long)blockIdx.x * DG_WARPS + (threadIdx.x >> 5);
+  if constexpr (ST)
+    if (q0 < tiles) sg.ask(Place<NI>(q0, L, rows), U);
+  load_coef(ga, reinterpret_cast<double2*>(sums), st->gamma, L);
+  Gr gr;
+  gr.init(&sums[0][threadIdx.x], outs[threadIdx.x >> 5]);
+  for (long long q = q0; q < tiles; q += step) {
+    const Place<NI> pl(q, L, rows);
+    double2 u[2][NI], v[2][NI];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int i = 0; i < NI; ++i) v[h][i] = make_double2(0.0, 0.0);
+#pragma unroll 1                           // one copy of the product's code: two overflow the instruction cache
+    for (int c = 0; c < 2; ++c) {
+      const double* base = c ? W : R;
+      double* out = c ? V : P;
+      if constexpr (ST) {
+        sg.take(u);
+        sg.ask(pl, c ? Rt : Y);
+      } else {
+        pl.load(c ? Y : U, u);
+      }
+      row_product<NI, ND>(
+          u, ga,
+          [&](int h, int nt) { return pl.ok(h, nt) ? at(base, pl.e[h] + 4 * nt) : make_double2(0.0, 0.0); },
+          [&](int h, int nt, double2 w, double2 p) {
+            if (!pl.ok(h, nt)) return;
+            const double2 x = make_double2(w.x + p.x, w.y + p.y);
+            at(out, pl.e[h] + 4 * nt) = x;
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+              if (i == nt) v[h][i] = x;    // V's in the end
+          });
+    }
+    if constexpr (ST) {
+      sg.take(u);
+      if (q + step < tiles) sg.ask(Place<NI>(q + step, L, rows), U);
+    } else {
+      pl.load(Rt, u);
+    }
+    gr.tile(u, v);
+  }
+  gr.write(part, outs[0], nullptr, L, nullptr);
+}
+
+// Calls f with the kernels' NI and ND.  Seven digits have the error of an FP64 sum from L = 4 on: relative to
+// U's rms, rms 1.23e-16 and largest 6.3e-16 at L = 4 (FP64 sums 1.19e-16 and 9.1e-16), 1.56e-16 and 9e-16 at
+// L = 12 on 8^4 (1.79e-16 and 1.6e-15); the shorter sums of FP64 mode take eight (L = 1: 0.79e-16,
+// against 0.93e-16 with seven and 0.83e-16 in FP64).  In the double-float updates seven are 30 times as exact
+// as the FP32 pairs were.
+template <class F>
+cudaError_t with_shape(int L, bool df, const F& f) {
+  using std::integral_constant;
+  if (L < 4 && !df) f(integral_constant<int, 1>(), integral_constant<int, 8>());
+  else if (L <= 4) f(integral_constant<int, 1>(), integral_constant<int, 7>());
+  else if (L <= 8) f(integral_constant<int, 2>(), integral_constant<int, 7>());
+  else if (L <= 12) f(integral_constant<int, 3>(), integral_constant<int, 7>());
+  else f(integral_constant<int, 4>(), integral_constant<int, 7>());
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_update_u_dg(const double* P, const double* V, double* U, int L, long long rows, int nb,
+                               const SolverState* st, cudaStream_t s, bool df) {
+  return with_shape(L, df, [&](auto ni, auto nd) {
+    update_u_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(P, V, U, L, rows, st);
+  });
+}
+
+cudaError_t launch_gram_dg(const double* A, const double* B, int L, long long rows, int nb, double2* part,
+                           bool norms, cudaStream_t s) {
+  return with_shape(L, false, [&](auto ni, auto nd) {
+    gram_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(A, B, L, rows, part, norms);
+  });
+}
+
+cudaError_t launch_update_xr_dg(double* X, const double* F, const double* G, double* R, const double* W,
+                                const double* Y, const double* Rt, int L, long long rows, int nb,
+                                double2* part, const SolverState* st, cudaStream_t s, bool df) {
+  return with_shape(L, df, [&](auto ni, auto nd) {
+    update_xr_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(X, F, G, R, W, Y, Rt, L, rows, part, st);
+  });
+}
+
+cudaError_t launch_update_pv_dg(double* P, double* V, const double* R, const double* W, const double* U,
+                                const double* Y, const double* Rt, int L, long long rows, int nb,
+                                double2* part, const SolverState* st, cudaStream_t s, bool df) {
+  return with_shape(L, df, [&](auto ni, auto nd) {
+    update_pv_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(P, V, R, W, U, Y, Rt, L, rows, part, st);
+  });
+}

@@ -156,6 +156,18 @@ int ts_max_blocks();             // largest such grid on the current device (4 x
 // Which L x L result a gram pass writes.
 enum { GRAM_RTR = 0, GRAM_RTR_NEW = 1, GRAM_RTV = 2 };
 
+// The three updates and the Gram products, products in exact digits on the tensor cores (blas_digits.cu); nb: grid size,
+// at most ts_max_blocks().
+cudaError_t launch_update_u_dg(const double* P, const double* V, double* U, int L, long long rows, int nb,
+                               const SolverState* st, cudaStream_t s, bool df);
+cudaError_t launch_gram_dg(const double* A, const double* B, int L, long long rows, int nb, double2* part,
+                           bool norms, cudaStream_t s);
+cudaError_t launch_update_xr_dg(double* X, const double* F, const double* G, double* R, const double* W,
+                                const double* Y, const double* Rt, int L, long long rows, int nb,
+                                double2* part, const SolverState* st, cudaStream_t s, bool df);
+cudaError_t launch_update_pv_dg(double* P, double* V, const double* R, const double* W, const double* U,
+                                const double* Y, const double* Rt, int L, long long rows, int nb,
+                                double2* part, const SolverState* st, cudaStream_t s, bool df);
 cudaError_t launch_gram(const double* A, const double* B, int L, long long rows, double2* part,
                         SolverState* st, int which, bool norms_of_b, cudaStream_t s);
 cudaError_t launch_colnorms(const double* A, int L, long long rows, double2* part,
