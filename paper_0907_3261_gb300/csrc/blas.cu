@@ -133,82 +133,118 @@ void finalize(const double2* part, int nblocks, int L, SolverState* st, int whic
   finalize_kernel<<<grid, FIN_COLS * FIN_ROWS, 0, s>>>(part, nblocks, L, st, which, norms_out, traces);
 }
 
-// ---------------------------------------------------------------- L x L solves (one warp)
-// Solves C Z = Rhs in place: M is the augmented L x 2L matrix [C | Rhs] in shared memory,
-// row-major with leading dimension 2*WD_LMAX.  Partial pivoting by the largest modulus.  Returns
-// true when the system is singular in the sense of the oracle: a pivot that is not finite or whose
-// modulus is below 1e-13 times the largest pivot modulus.
-constexpr double PIVOT_RTOL = 1e-13;
-constexpr int LD = 2 * WD_LMAX;
+// ---------------------------------------------------------------- L x L solves (one block)
+// Solves C Z = Rhs by elimination with partial pivoting (largest modulus) and back substitution.  Thread
+// e < 2 L^2 holds element (i, j) = (e % L, e / L) of [C | Rhs]; rows are not moved, a row's place in the pivots'
+// order is kept instead.  A warp's FP64 instruction takes 64 cycles of its quarter of the SM whatever its
+// lanes do, so the count per warp is what bounds the solve: elements are dense in the warps, moduli are
+// compared as integers, and the column's owners alone form the pivot's reciprocal and the factors.  27 us at
+// L = 12 and 8 at L = 4, against about 75 and 18 in one warp with a column per lane; an iteration of a 4^4,
+// L = 12 solve 256 us against 353.
+//
+// The system is singular in the sense of the oracle when a pivot is not finite or its modulus is below
+// 1e-13 times the largest pivot's.
+constexpr double PIVOT_RTOL2 = 1e-26;      // squared moduli are compared
 
-__device__ bool lu_solve_warp(Cx<double>* M, int L) {
-  const int lane = threadIdx.x;
-  double pmax = 0.0, pmin = 1e308;
-  bool bad = false;
+struct Lu {
+  double2 u[WD_LMAX][2 * WD_LMAX];         // the pivot rows, in their order
+  double2 c[WD_LMAX], f[WD_LMAX];          // a column, its factors
+  double2 rp[WD_LMAX];                     // the pivots' reciprocals
+  double2 x[WD_LMAX];                      // a row of the solution
+  long long norm[WD_LMAX];                 // bits of the squared moduli, -1 for rows that have been pivots
+  double pn[WD_LMAX];
+  double2 extra;                           // a number that the block's last warp computes beside
+};
+
+inline int lu_threads(int L) { return (2 * L * L + 31) / 32 * 32 + 32; }
+
+// m: this thread's element (i, j).  On return `order` is row i's place and, for j >= L, m the solution's element
+// (order, j - L).  The same in every thread: true when the system is singular (`order` may then be L).
+__device__ bool lu_solve(Lu& s, Cx<double>& m, int L, int i, int j, bool live, int& order) {
+  order = L;                               // not yet a pivot
   for (int k = 0; k < L; ++k) {
-    int p = k;
-    double best = cnorm2(M[k * LD + k]);
-    for (int i = k + 1; i < L; ++i) {
-      const double v = cnorm2(M[i * LD + k]);
-      if (v > best) { best = v; p = i; }
+    if (live && j == k) {
+      s.c[i] = d2(m);
+      s.norm[i] = order < L ? -1 : __double_as_longlong(cnorm2(m));
     }
-    __syncwarp();
-    if (p != k && lane < 2 * L) {
-      const Cx<double> tmp = M[k * LD + lane];
-      M[k * LD + lane] = M[p * LD + lane];
-      M[p * LD + lane] = tmp;
+    __syncthreads();
+    int p = 0;
+    long long best = -2;
+    for (int q = 0; q < L; ++q) {
+      const long long v = s.norm[q];
+      if (v > best) {
+        best = v;
+        p = q;
+      }
     }
-    __syncwarp();
-    const Cx<double> piv = M[k * LD + k];
-    const double pa = sqrt(cnorm2(piv));
-    if (!isfinite(pa) || pa == 0.0) bad = true;
-    pmax = fmax(pmax, pa);
-    pmin = fmin(pmin, pa);
-    const double pn = cnorm2(piv);
-    const Cx<double> rp = cmake(piv.re / pn, -piv.im / pn);
-    for (int i = k + 1; i < L; ++i) {
-      const Cx<double> f = cmul(M[i * LD + k], rp);
-      __syncwarp();
-      if (lane > k && lane < 2 * L) M[i * LD + lane] = M[i * LD + lane] - cmul(f, M[k * LD + lane]);
-      if (lane == k) M[i * LD + k] = f;
-      __syncwarp();
+    const bool mine = live && i == p;
+    if (mine) {
+      order = k;
+      s.u[k][j] = d2(m);
     }
-  }
-  if (!(pmin >= PIVOT_RTOL * pmax)) bad = true;
-  // back substitution, one right-hand-side column per lane
-  if (lane >= L && lane < 2 * L) {
-    for (int i = L - 1; i >= 0; --i) {
-      Cx<double> v = M[i * LD + lane];
-      for (int jj = i + 1; jj < L; ++jj) v = v - cmul(M[i * LD + jj], M[jj * LD + lane]);
-      const Cx<double> d = M[i * LD + i];
-      const double dn = cnorm2(d);
-      M[i * LD + lane] = cmul(v, cmake(d.re / dn, -d.im / dn));
+    if (live && j == k) {
+      const double pn = __longlong_as_double(best), r = 1.0 / pn;
+      const Cx<double> rp = cmake(s.c[p].x * r, -s.c[p].y * r);
+      if (mine) {
+        s.rp[k] = d2(rp);
+        s.pn[k] = pn;
+      }
+      s.f[i] = d2(cmul(m, rp));            // the factor of row i (of no use in the pivot's)
+    }
+    __syncthreads();
+    if (live && order == L && j > k) {
+      const double2 f = s.f[i], u = s.u[k][j];
+      m.re = fma(f.y, u.y, fma(-f.x, u.x, m.re));
+      m.im = fma(-f.y, u.x, fma(-f.x, u.y, m.im));
     }
   }
-  __syncwarp();
+  long long lo = 0x7FFFFFFFFFFFFFFFll, hi = 0;
+  for (int k = 0; k < L; ++k) {
+    const long long v = __double_as_longlong(s.pn[k]);
+    lo = min(lo, v);
+    hi = max(hi, v);
+  }
+  const bool bad = hi >= 0x7FF0000000000000ll || lo <= 0 ||
+                   !(__longlong_as_double(lo) >= PIVOT_RTOL2 * __longlong_as_double(hi));
+  const bool rhs = live && j >= L;
+  for (int k = L - 1; k >= 0; --k) {
+    if (rhs && order == k) {
+      m = cmul(m, sm(s.rp[k]));
+      s.x[j - L] = d2(m);
+    }
+    __syncthreads();
+    if (rhs && order < k) {
+      const double2 u = s.u[order][k], x = s.x[j - L];
+      m.re = fma(u.y, x.y, fma(-u.x, x.x, m.re));
+      m.im = fma(-u.y, x.x, fma(-u.x, x.y, m.im));
+    }
+    __syncthreads();
+  }
   return bad;
 }
 
 // alpha_k from (R~_0^H V_k) alpha_k = R~_0^H R_k, and zeta_k = Tr[W^H R] / Tr[W^H W].
 __global__ void solve_alpha_kernel(SolverState* st, int L) {
-  __shared__ Cx<double> M[WD_LMAX * LD];
+  __shared__ Lu s;
   if (st->status != ST_OK) return;
-  const int lane = threadIdx.x;
-  for (int i = 0; i < L; ++i)
-    if (lane < L) {
-      M[i * LD + lane] = sm(st->rtv[i * L + lane]);
-      M[i * LD + L + lane] = sm(st->rtr[i * L + lane]);
-    }
-  __syncwarp();
-  const bool bad = lu_solve_warp(M, L);
-  if (lane < L)
-    for (int i = 0; i < L; ++i) st->alpha[i * L + lane] = bad ? make_double2(0, 0) : d2(M[i * LD + L + lane]);
-  if (lane == 0) {
+  const int e = threadIdx.x, j = e / L, i = e - j * L;
+  const bool live = j < 2 * L;
+  if (e == blockDim.x - 32) {
     const double ww = st->trww;
-    const Cx<double> wr = sm(st->trwr);
-    Cx<double> z = cmake(wr.re / ww, wr.im / ww);
-    bool zbad = !(ww > 0.0) || !isfinite(z.re) || !isfinite(z.im);
-    st->zeta = zbad ? make_double2(0, 0) : d2(z);
+    const double2 wr = st->trwr;
+    const double2 z = make_double2(wr.x / ww, wr.y / ww);
+    // an imaginary part of NaN marks a zeta that cannot be used
+    const bool bad = !(ww > 0.0) || !isfinite(z.x) || !isfinite(z.y);
+    s.extra = bad ? make_double2(0.0, __longlong_as_double(0x7FF8000000000000ll)) : z;
+  }
+  Cx<double> m = czero<double>();
+  if (live) m = j < L ? sm(st->rtv[i * L + j]) : sm(st->rtr[i * L + j - L]);
+  int row;
+  const bool bad = lu_solve(s, m, L, i, j, live, row);
+  if (live && j >= L) st->alpha[(bad ? i : row) * L + j - L] = bad ? make_double2(0, 0) : d2(m);
+  if (e == 0) {
+    const bool zbad = isnan(s.extra.y);
+    st->zeta = zbad ? make_double2(0, 0) : s.extra;
     if (bad) st->status = ST_ALPHA_SINGULAR;
     else if (zbad) st->status = ST_ZETA_BAD;
   }
@@ -216,25 +252,27 @@ __global__ void solve_alpha_kernel(SolverState* st, int L) {
 
 // gamma_k from (R~_0^H R_k) gamma_k = R~_0^H R_{k+1} / zeta_k; then R~_0^H R_k <- R~_0^H R_{k+1}.
 __global__ void solve_gamma_kernel(SolverState* st, int L) {
-  __shared__ Cx<double> M[WD_LMAX * LD];
+  __shared__ Lu s;
   if (st->status != ST_OK) return;
-  const int lane = threadIdx.x;
-  const Cx<double> z = sm(st->zeta);
-  const double zn = cnorm2(z);
-  const Cx<double> rz = cmake(z.re / zn, -z.im / zn);
-  for (int i = 0; i < L; ++i)
-    if (lane < L) {
-      M[i * LD + lane] = sm(st->rtr[i * L + lane]);
-      M[i * LD + L + lane] = cmul(sm(st->rtr_new[i * L + lane]), rz);
-    }
-  __syncwarp();
-  const bool bad = lu_solve_warp(M, L);
-  if (lane < L)
-    for (int i = 0; i < L; ++i) {
-      st->gamma[i * L + lane] = bad ? make_double2(0, 0) : d2(M[i * LD + L + lane]);
-      st->rtr[i * L + lane] = st->rtr_new[i * L + lane];
-    }
-  if (lane == 0 && bad) st->status = ST_GAMMA_SINGULAR;
+  const int e = threadIdx.x, j = e / L, i = e - j * L;
+  const bool live = j < 2 * L;
+  if (e == blockDim.x - 32) {
+    const double2 z = st->zeta;
+    const double r = 1.0 / (z.x * z.x + z.y * z.y);
+    s.extra = make_double2(z.x * r, -z.y * r);
+  }
+  Cx<double> m = czero<double>();
+  if (live) m = j < L ? sm(st->rtr[i * L + j]) : sm(st->rtr_new[i * L + j - L]);
+  const Cx<double> next = m;
+  __syncthreads();
+  if (live && j >= L) m = cmul(m, sm(s.extra));
+  int row;
+  const bool bad = lu_solve(s, m, L, i, j, live, row);
+  if (live && j >= L) {
+    st->gamma[(bad ? i : row) * L + j - L] = bad ? make_double2(0, 0) : d2(m);
+    st->rtr[i * L + j - L] = d2(next);
+  }
+  if (e == 0 && bad) st->status = ST_GAMMA_SINGULAR;
 }
 
 // Four blocks of TS_THREADS per SM, for the current device (its SM count is read once per device).
@@ -300,12 +338,12 @@ cudaError_t launch_traces(const double* W, const double* R, int L, long long row
 }
 
 cudaError_t launch_solve_alpha(SolverState* st, int L, cudaStream_t s) {
-  solve_alpha_kernel<<<1, 32, 0, s>>>(st, L);
+  solve_alpha_kernel<<<1, lu_threads(L), 0, s>>>(st, L);
   return cudaGetLastError();
 }
 
 cudaError_t launch_solve_gamma(SolverState* st, int L, cudaStream_t s) {
-  solve_gamma_kernel<<<1, 32, 0, s>>>(st, L);
+  solve_gamma_kernel<<<1, lu_threads(L), 0, s>>>(st, L);
   return cudaGetLastError();
 }
 
