@@ -463,7 +463,7 @@ sweep_df2_kernel(const float4* __restrict__ x, TY* __restrict__ y, const float4*
 // product rounded to the grid, with no other rounding, and fma(a, b.hi, S - S') -- S - S' is exact
 // -- is the part of the product below the grid, |.| <= g/2, rounded to 24 bits of itself.  That
 // part and a b.lo go into a plain FP32 sum.  Per product: 5 FP32x2 operations instead of 11, at an
-// error of ~2^-24 g per product instead of an exact high part (see DESIGN: the sum's error stays
+// error of ~2^-24 g per product instead of an exact high part (the sum's error stays
 // ~2^-44 of the bound, the order of the two-sum form's low-word rounding).
 //   Bounds.  A hop sums three products of a link row (norm <= 1: op.links_unitary) with the
 // projected half-spinor h, so each partial sum is below sqrt(3) m, m = max |h.hi| over the hop's
