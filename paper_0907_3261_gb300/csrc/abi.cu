@@ -735,10 +735,6 @@ void wd_destroy(wd_ctx* c) {
   cudaFree(c->op.links32s);
   cudaFree(c->op.clov_inv32s);
   cudaFree(c->op.fx_links);
-  cudaFree(c->op.fx_clov);
-  cudaFree(c->op.fx_cinv);
-  cudaFree(c->op.fx_nb);
-  cudaFree(c->op.fx_exps);
   c->field.release();
   for (auto& b : c->blk) b.release();
   for (auto& b : c->blk32) b.release();
@@ -788,11 +784,12 @@ static int create_impl(wd_ctx* c, const void* links, const int dims[4], cudaStre
     return WD_BREAKDOWN;
   }
   if (op.links_unitary) {   // the fixed-point form of the FP64 stencil (its bounds need unitary links)
-    CU(cudaMalloc(&op.fx_links, V * FX_WSTR * sizeof(int4)));
-    CU(cudaMalloc(&op.fx_clov, V * FX_DSTR * sizeof(int4)));
-    CU(cudaMalloc(&op.fx_cinv, V * FX_DSTR * sizeof(int4)));
-    CU(cudaMalloc(&op.fx_nb, V * 2 * sizeof(int4)));
-    CU(cudaMalloc(&op.fx_exps, 3 * V * WD_LMAX * sizeof(short)));
+    // one block: an allocation costs as much as building a small lattice's tables
+    CU(cudaMalloc(&op.fx_links, V * ((FX_WSTR + 2 * FX_DSTR + 2) * sizeof(int4) + 3 * WD_LMAX * sizeof(short))));
+    op.fx_clov = op.fx_links + V * FX_WSTR;
+    op.fx_cinv = op.fx_clov + V * FX_DSTR;
+    op.fx_nb = op.fx_cinv + V * FX_DSTR;
+    op.fx_exps = reinterpret_cast<short*>(op.fx_nb + V * 2);
     op.fx_ek = fx_link_exponent(op.kappa);
     CU(launch_fx_tables(op, s));
     CU(cudaStreamSynchronize(s));
