@@ -176,7 +176,6 @@ WD_DEV DF df_norm(DF a) {
 struct CDF {
   DF re, im;
 };
-WD_DEV CDF cdf_from(Cx<double> z) { return {df_from(z.re), df_from(z.im)}; }
 WD_DEV Cx<double> cdf_to(CDF z) { return {df_to(z.re), df_to(z.im)}; }
 WD_DEV CDF cdf_split(Cx<double> z) { return {df_split(z.re), df_split(z.im)}; }
 WD_DEV Cx<double> cdf_join(CDF z) { return {df_join(z.re), df_join(z.im)}; }
@@ -226,33 +225,10 @@ WD_DEV P2 padd(P2 a, P2 b, float2 sg, float2 m1) {   // a + sg b
 }
 // (re, im) = X + (-Y.im, Y.re): sum a_k b_k from its two accumulators.
 WD_DEV P2 pcombine(P2 X, P2 Y, float2 m1) { return padd(X, pswap(Y), make_float2(-1.f, 1.f), m1); }
-// (re, im) = X + (Y.im, -Y.re): sum conj(a_k) b_k from its two accumulators.
-WD_DEV P2 pcombine_conj(P2 X, P2 Y, float2 m1) {
-  return padd(X, pswap(Y), make_float2(1.f, -1.f), m1);
-}
-// hi + lo renormalised so that |lo| <= ulp(hi)/2, in both lanes.
-WD_DEV P2 pnorm(P2 z, float2 m1) {
-  const float2 s = __fadd2_rn(z.hi, z.lo);
-  return {s, __ffma2_rn(__ffma2_rn(z.hi, m1, s), m1, z.lo)};   // lo - (s - hi)
-}
-// acc + a b for a double-float factor a = ahi + alo given per lane (nahi = -ahi), b packed.
-WD_DEV void pmac_dd(P2& acc, float2 ahi, float2 nahi, float2 alo, P2 b, float2 m1) {
-  const float2 np = __fmul2_rn(nahi, b.hi);   // -(ahi b.hi), rounded
-  float2 e = __ffma2_rn(ahi, b.hi, np);       // its rounding error, exactly
-  e = __ffma2_rn(ahi, b.lo, e);
-  e = __ffma2_rn(alo, b.hi, e);
-  float2 s, t;
-  two_sum2(acc.hi, np, m1, m1, s, t);         // acc.hi - np
-  acc.hi = s;
-  acc.lo = __fadd2_rn(acc.lo, __fadd2_rn(t, e));
-}
-// FP64 (re, im) <-> packed double-float through the bit-field conversions.
+// FP64 (re, im) to packed double-float through the bit-field conversion.
 WD_DEV P2 p2_split(double2 v) {
   const DF r = df_split(v.x), i = df_split(v.y);
   return {make_float2(r.hi, i.hi), make_float2(r.lo, i.lo)};
-}
-WD_DEV double2 p2_join(P2 z) {   // one FP64 rounding of hi + lo per lane
-  return make_double2(f_widen(z.hi.x) + f_widen(z.lo.x), f_widen(z.hi.y) + f_widen(z.lo.y));
 }
 
 // ------------------------------------------------------------------ grid sums (packed)
