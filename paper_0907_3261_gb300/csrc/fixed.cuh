@@ -106,10 +106,12 @@ WD_DEV int neighbours_and_scale(const int4* __restrict__ nbt, const short* __res
 // The sums of this thread's chirality from the hops' sums: the even thread of a pair takes the upper
 // chirality, so both threads' upper spins; the odd one the lower: for spin 2 its own through mu 0, 1 and
 // the other's through mu 2, 3, for spin 3 the reverse.  acc: [2][6][TPB] lower sums through mu 0, 1 and
-// mu 2, 3, overwritten by the odd thread; hs: components (spin, colour, re/im).
+// mu 2, 3, overwritten by the odd thread; hs: components (spin, colour, re/im).  Begins with a barrier of
+// the warp: the other thread's slots are read, and nothing before makes its last sums visible.
 template <typename T>
 WD_DEV void exchange(T (*acc)[6][TPB], const T au[6], int sp, T hs[12]) {
   const int t = threadIdx.x, o = t ^ 1;
+  __syncwarp();
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
     const T a = acc[0][q][t], b = acc[1][q][t], c = acc[1][q][o], d = acc[0][q][o];
