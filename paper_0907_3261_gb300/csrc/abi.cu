@@ -119,8 +119,11 @@ struct wd_ctx {
   DevBuf stage_in, stage_out;
   // low-precision preconditioner blocks: U and two sweep buffers (sized for FP32 elements)
   DevBuf blk32[3];
-  // the copy of a product's operand in the fixed-point stencil's form (one block)
+  // the copy of a product's operand in the fixed-point stencil's form (one block), whether a captured
+  // product uses it, and outgrown blocks that captured products use
   DevBuf field;
+  bool field_captured = false;
+  std::vector<DevBuf> captured_fields;
   // autotuned tile of the low-precision sweep per storage (LP_F32, LP_BF16, LP_DF) and L: RHS per
   // thread, threads per CTA, min CTAs per SM, shared-memory staging
   int tile_r[3][WD_LMAX + 1] = {};
@@ -256,24 +259,34 @@ int ensure_workspace(wd_ctx* c, int L) {
 // The block for the fixed-point stencil's copy of its operand, allocated at the first product with an L
 // (grown, never shrunk).  Null -- the product then runs on the FP64 pipe, which needs no
 // memory -- when the form is not in use, when the device has no room for the block, or when it would
-// have to be allocated while `s` is being captured.
+// have to be allocated while `s` is being captured.  A graph that a capture of a product made holds the
+// block's address: an outgrown block is then kept until wd_destroy.
 void* field_block(wd_ctx* c, int L, cudaStream_t s) {
   if (c->op.apply_form != 1) return nullptr;
   const size_t bytes = block_bytes(c, L);
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
   if (c->field.bytes < bytes) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    if (capturing) return nullptr;
+    DevBuf grown;
+    cudaError_t e = cudaMalloc(&grown.p, bytes);
+    if (e != cudaSuccess && c->field.p && !c->field_captured) {   // no room for both
+      cudaGetLastError();
+      c->field.release();
+      e = cudaMalloc(&grown.p, bytes);
+    }
+    if (e != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
-    c->field.release();
-    if (cudaMalloc(&c->field.p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      c->field.p = nullptr;
-      return nullptr;
-    }
-    c->field.bytes = bytes;
+    grown.bytes = bytes;
+    if (c->field_captured) c->captured_fields.push_back(c->field);
+    else c->field.release();
+    c->field = grown;
+    c->field_captured = false;
   }
+  c->field_captured = c->field_captured || capturing;
   return c->field.p;
 }
 
@@ -736,6 +749,7 @@ void wd_destroy(wd_ctx* c) {
   cudaFree(c->op.clov_inv32s);
   cudaFree(c->op.fx_links);
   c->field.release();
+  for (auto& b : c->captured_fields) b.release();
   for (auto& b : c->blk) b.release();
   for (auto& b : c->blk32) b.release();
   c->part.release();
