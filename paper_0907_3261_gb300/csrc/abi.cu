@@ -256,8 +256,8 @@ int ensure_workspace(wd_ctx* c, int L) {
   return WD_OK;
 }
 
-// The block for the fixed-point stencil's copy of its operand, allocated at the first product with an L
-// (grown, never shrunk).  Null -- the product then runs on the FP64 pipe, which needs no
+// The block for the copy of a product's operand that the fixed-point stencil takes (wd_apply; a solve uses
+// its own scratch), allocated at the first product with an L (grown, never shrunk).  Null -- the product then runs on the FP64 pipe, which needs no
 // memory -- when the form is not in use, when the device has no room for the block, or when it would
 // have to be allocated while `s` is being captured.  A graph that a capture of a product made holds the
 // block's address: an outgrown block is then kept until wd_destroy.
@@ -617,12 +617,13 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
   double* pT = c->blk[B_T].d();
   double2* part = static_cast<double2*>(c->part.p);
   SolverState* st = c->st;
-  void* const field = field_block(c, L, s);
+  // The product's copy of its operand goes to the preconditioner's scratch block, free at every product.
+  auto field = [&]() -> void* { return op.apply_form == 1 ? pT : nullptr; };
   CU(cudaMemsetAsync(&st->status, 0, sizeof(int), s));
 
   // R_0 = B - A X_0;  P_0 = R_0;  R~_0 = R_0
   CHECK(halo_exchange(c, X, L, s));
-  LAUNCH(WD_K_RESID, stencil_kernels(op, field), launch_resid_f64(op, X, B, R, field, L, s));
+  LAUNCH(WD_K_RESID, stencil_kernels(op, field()), launch_resid_f64(op, X, B, R, field(), L, s));
   ++*hop_count;
   LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(P, R, bytes, cudaMemcpyDeviceToDevice, s));
   LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(Rt, R, bytes, cudaMemcpyDeviceToDevice, s));
@@ -641,7 +642,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
   CHECK(precondition(c, R, pF, pT, &res, L, j, precision, hop_count, s));
   if (res != pF) { pT = pF; pF = res; }
   CHECK(halo_exchange(c, pF, L, s));
-  LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, pF, W, field, L, s));
+  LAUNCH(WD_K_APPLY, stencil_kernels(op, field()), launch_apply_f64(op, pF, W, field(), L, s));
   ++*hop_count;
   LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(V, W, bytes, cudaMemcpyDeviceToDevice, s));
   LAUNCH(WD_K_TRACE, 2, launch_traces(in(W), in(R), L, rows, part, st, s));
@@ -660,7 +661,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
     CHECK(precondition(c, U, pG, pT, &res, L, j, precision, hop_count, s));   // G_k = M U_k
     if (res != pG) { pT = pG; pG = res; }
     CHECK(halo_exchange(c, pG, L, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, pG, Y, field, L, s));                  // Y_k = A G_k
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field()), launch_apply_f64(op, pG, Y, field(), L, s));                  // Y_k = A G_k
     ++*hop_count;
     LAUNCH(WD_K_UPDATE_XR, 2, launch_update_xr(in(X), cin(pF), cin(pG), in(R), cin(W), cin(Y), cin(Rt), L, rows, part, st, s, df));   // X_{k+1}, R_{k+1}
     CHECK(dom_sum(c, st->rtr_new, 2 * L * L, s));
@@ -678,7 +679,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
     CHECK(precondition(c, R, pF, pT, &res, L, j, precision, hop_count, s));   // F_{k+1} = M R_{k+1}
     if (res != pF) { pT = pF; pF = res; }
     CHECK(halo_exchange(c, pF, L, s));
-    LAUNCH(WD_K_APPLY, stencil_kernels(op, field), launch_apply_f64(op, pF, W, field, L, s));                  // W_{k+1} = A F_{k+1}
+    LAUNCH(WD_K_APPLY, stencil_kernels(op, field()), launch_apply_f64(op, pF, W, field(), L, s));                  // W_{k+1} = A F_{k+1}
     ++*hop_count;
     LAUNCH(WD_K_TRACE, 2, launch_traces(in(W), in(R), L, rows, part, st, s));  // Tr[W^H R], Tr[W^H W]
     CHECK(dom_sum(c, &st->trwr, 3, s));
@@ -1235,7 +1236,7 @@ int bbicggr_solve(wd_ctx* c, const void* B, void* X, int L, int j, double tol,
     if (rr.status == RUN_STALLED) rr.status = WD_NOT_CONVERGED;
     // true residual ||b_i - A x_i|| / ||b_i||
     double* T = c->blk[B_T].d();
-    void* const field = field_block(c, L, s);
+    void* const field = c->op.apply_form == 1 ? c->blk[B_W].p : nullptr;   // W is not needed any more
     CHECK(halo_exchange(c, Xd, L, s));
     LAUNCH(WD_K_RESID, stencil_kernels(c->op, field), launch_resid_f64(c->op, Xd, Bd, T, field, L, s));
     ++hops;
@@ -1476,7 +1477,7 @@ int build_run(wd_ctx* c, const JobPtrs& jp, int mode, bool df, bool restore, cud
   SolverState* st = c->st;
   GraphCtl* g = static_cast<GraphCtl*>(c->gctl);
   double* hist = c->ghist;
-  void* const field = c->op.apply_form == 1 ? c->field.p : nullptr;
+  void* const field = op.apply_form == 1 ? T : nullptr;   // free at every product (run_bbicggr)
 
   cudaGraphConditionalHandle hloop;
   CU(cudaGraphConditionalHandleCreate(&hloop, RB, 0, 0));
@@ -1565,7 +1566,7 @@ int build_job(wd_ctx* c, const JobPtrs& jp, cudaGraph_t G) {
   double2* part = static_cast<double2*>(c->part.p);
   GraphCtl* g = static_cast<GraphCtl*>(c->gctl);
   const bool two_modes = jp.X0 != nullptr;
-  void* const field = op.apply_form == 1 ? c->field.p : nullptr;
+  void* const field = op.apply_form == 1 ? c->blk[B_W].p : nullptr;   // W is not needed any more
 
   cudaGraphConditionalHandle hphase;
   CU(cudaGraphConditionalHandleCreate(&hphase, G, 1, cudaGraphCondAssignDefault));
@@ -1635,7 +1636,6 @@ extern "C" int bbicggr_solve_batch(bbicggr_job* jobs, int njobs, void* stream) {
     bbicggr_job& jb = jobs[i];
     wd_ctx* c = jb.ctx;
     CHECK(ensure_workspace(c, jb.L));
-    field_block(c, jb.L, s);
     const int mode = precond_mode(jb.opts);
     if ((mode == PM_F32 || mode == PM_BF16) && jb.j >= 2)
       CHECK(ensure_workspace_lp(c, lp_storage(mode), jb.L, s));
