@@ -124,6 +124,11 @@ struct wd_ctx {
   DevBuf field;
   bool field_captured = false;
   std::vector<DevBuf> captured_fields;
+  // ... and the block for small operands, part of the operator tables' allocation; in use from the first
+  // product outside a capture
+  void* small_field = nullptr;
+  size_t small_field_bytes = 0;
+  bool small_field_used = false;
   // autotuned tile of the low-precision sweep per storage (LP_F32, LP_BF16, LP_DF) and L: RHS per
   // thread, threads per CTA, min CTAs per SM, shared-memory staging
   int tile_r[3][WD_LMAX + 1] = {};
@@ -256,17 +261,33 @@ int ensure_workspace(wd_ctx* c, int L) {
   return WD_OK;
 }
 
+// An allocation costs 80 to 130 us, so a context's first product was slower than in FP32 sums (4^4, L = 12:
+// 143 us against 80; 8^4: 145 against 118; 12^3x24, L = 1: 171 against 160; 8^3x16, L = 12, 19 MB: equal at
+// 175).  Copies up to this size have their place from the creation of the context on.
+constexpr size_t SMALL_FIELD_MAX = (size_t)24 << 20;
+size_t small_field_bytes(long long V) {
+  const size_t column = (size_t)V * 12 * 16;
+  return column > SMALL_FIELD_MAX ? 0 : std::min(column * WD_LMAX, SMALL_FIELD_MAX / 16 * 16);
+}
+
 // The block for the copy of a product's operand that the fixed-point stencil takes (wd_apply; a solve uses
-// its own scratch), allocated at the first product with an L (grown, never shrunk).  Null -- the product then runs on the FP64 pipe, which needs no
+// its own scratch): the context's for small operands, or one allocated at the first product with an L
+// (grown, never shrunk).  Null -- the product then runs on the FP64 pipe, which needs no
 // memory -- when the form is not in use, when the device has no room for the block, or when it would
 // have to be allocated while `s` is being captured.  A graph that a capture of a product made holds the
-// block's address: an outgrown block is then kept until wd_destroy.
+// block's address: an outgrown block is then kept until wd_destroy.  (A capture before the first product
+// runs on the FP64 pipe for small operands too: what it computes does not depend on their size.)
 void* field_block(wd_ctx* c, int L, cudaStream_t s) {
   if (c->op.apply_form != 1) return nullptr;
   const size_t bytes = block_bytes(c, L);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   const bool capturing = cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
   cudaGetLastError();
+  if (bytes <= c->small_field_bytes) {
+    if (capturing && !c->small_field_used) return nullptr;
+    c->small_field_used = true;
+    return c->small_field;
+  }
   if (c->field.bytes < bytes) {
     if (capturing) return nullptr;
     DevBuf grown;
@@ -800,7 +821,10 @@ static int create_impl(wd_ctx* c, const void* links, const int dims[4], cudaStre
   }
   if (op.links_unitary) {   // the fixed-point form of the FP64 stencil (its bounds need unitary links)
     // one block: an allocation costs as much as building a small lattice's tables
-    CU(cudaMalloc(&op.fx_links, V * ((FX_WSTR + 2 * FX_DSTR + 2) * sizeof(int4) + 3 * WD_LMAX * sizeof(short))));
+    const size_t tables = V * ((FX_WSTR + 2 * FX_DSTR + 2) * sizeof(int4) + 3 * WD_LMAX * sizeof(short));
+    c->small_field_bytes = small_field_bytes(V);
+    CU(cudaMalloc(&op.fx_links, tables + c->small_field_bytes));
+    c->small_field = reinterpret_cast<char*>(op.fx_links) + tables;
     op.fx_clov = op.fx_links + V * FX_WSTR;
     op.fx_cinv = op.fx_clov + V * FX_DSTR;
     op.fx_nb = op.fx_cinv + V * FX_DSTR;
