@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <initializer_list>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/bbicggr.h"
@@ -124,7 +125,10 @@ struct wd_ctx {
   DevBuf field;
   bool field_captured = false;
   std::vector<DevBuf> captured_fields;
-  // ... and the block for small operands, part of the operator tables' allocation; in use from the first
+  // the operator and its tables (c->op points into them), the fixed-point tables of a large lattice
+  void* arena = nullptr;
+  void* tables = nullptr;
+  // the place for the copy of a small operand, part of the fixed-point tables' allocation; in use from the first
   // product outside a capture
   void* small_field = nullptr;
   size_t small_field_bytes = 0;
@@ -265,6 +269,9 @@ int ensure_workspace(wd_ctx* c, int L) {
 // 143 us against 80; 8^4: 145 against 118; 12^3x24, L = 1: 171 against 160; 8^3x16, L = 12, 19 MB: equal at
 // 175).  Copies up to this size have their place from the creation of the context on.
 constexpr size_t SMALL_FIELD_MAX = (size_t)24 << 20;
+// Fixed-point tables up to this size are part of the operator's allocation.
+constexpr size_t SMALL_TABLES_MAX = (size_t)64 << 20;
+constexpr size_t FX_SITE_BYTES = (FX_WSTR + 2 * FX_DSTR + 2) * sizeof(int4) + 3 * WD_LMAX * sizeof(short);
 size_t small_field_bytes(long long V) {
   const size_t column = (size_t)V * 12 * 16;
   return column > SMALL_FIELD_MAX ? 0 : std::min(column * WD_LMAX, SMALL_FIELD_MAX / 16 * 16);
@@ -761,15 +768,8 @@ void wd_destroy(wd_ctx* c) {
   if (!c) return;
   harvest(c);
   for (auto e : c->prof.pool) cudaEventDestroy(e);
-  cudaFree(c->op.links);
-  cudaFree(c->op.clov);
-  cudaFree(c->op.clov_inv);
-  cudaFree(c->op.links32);
-  cudaFree(c->op.clov_inv32);
-  cudaFree(c->op.clov_bound32);
-  cudaFree(c->op.links32s);
-  cudaFree(c->op.clov_inv32s);
-  cudaFree(c->op.fx_links);
+  cudaFree(c->arena);
+  cudaFree(c->tables);
   c->field.release();
   for (auto& b : c->captured_fields) b.release();
   for (auto& b : c->blk) b.release();
@@ -791,26 +791,38 @@ static int create_impl(wd_ctx* c, const void* links, const int dims[4], cudaStre
   Op& op = c->op;
   const size_t V = op.g.V;
   const size_t lbytes = V * 4 * 18 * sizeof(double);
-  CU(cudaMalloc(&op.links, lbytes));
-  CU(cudaMalloc(&op.clov, V * 2 * CLOV_REALS * sizeof(double)));
-  CU(cudaMalloc(&op.clov_inv, V * 2 * CLOV_REALS * sizeof(double)));
-  CU(cudaMalloc(&op.links32, V * 4 * 18 * sizeof(float)));
-  CU(cudaMalloc(&op.clov_inv32, V * 2 * CLOV_REALS * sizeof(float)));
-  CU(cudaMalloc(&op.clov_bound32, V * 2 * sizeof(float)));
-  CU(cudaMalloc(&op.links32s, V * 4 * 5 * sizeof(float4)));
-  CU(cudaMalloc(&op.clov_inv32s, V * 2 * (CLOV_REALS / 4) * sizeof(float4)));
+  // One allocation for the operator, and for a small lattice its fixed-point tables too (they need unitary
+  // links, which is not known yet).  flag [0]: a singular A_D block; [1]: a link that is not special unitary;
+  // [2]: a link with a row or column of norm above 1.
+  c->small_field_bytes = small_field_bytes(V);
+  const size_t tables = V * FX_SITE_BYTES + c->small_field_bytes;
+  const bool with_tables = tables <= SMALL_TABLES_MAX;
+  int* flag = nullptr;
+  for (int pass = 0; pass < 2; ++pass) {     // first the sizes, then the places
+    size_t used = 0;
+    auto take = [&](auto*& q, size_t bytes) {
+      if (pass) q = reinterpret_cast<std::remove_reference_t<decltype(q)>>(static_cast<char*>(c->arena) + used);
+      used += (bytes + 255) / 256 * 256;
+    };
+    take(op.links, lbytes);
+    take(op.clov, V * 2 * CLOV_REALS * sizeof(double));
+    take(op.clov_inv, V * 2 * CLOV_REALS * sizeof(double));
+    take(op.links32, V * 4 * 18 * sizeof(float));
+    take(op.clov_inv32, V * 2 * CLOV_REALS * sizeof(float));
+    take(op.clov_bound32, V * 2 * sizeof(float));
+    take(op.links32s, V * 4 * 5 * sizeof(float4));
+    take(op.clov_inv32s, V * 2 * (CLOV_REALS / 4) * sizeof(float4));
+    take(flag, 3 * sizeof(int));
+    if (with_tables) take(op.fx_links, tables);
+    if (!pass) CU(cudaMalloc(&c->arena, used));
+  }
   CU(cudaMemcpyAsync(op.links, links, lbytes, cudaMemcpyDefault, s));
-  // [0]: a singular A_D block; [1]: a link that is not special unitary; [2]: a link with a row or
-  // column of norm above 1
-  int* flag;
-  CU(cudaMalloc(&flag, 3 * sizeof(int)));
   CU(cudaMemsetAsync(flag, 0, 3 * sizeof(int), s));
   CU(launch_clover_build(op, flag, s));
   CU(launch_lp_operator_copies(op, flag + 1, s));
   int h[3] = {0, 0, 0};
   cudaError_t e = cudaMemcpyAsync(h, flag, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(flag);
   CU(e);
   c->links_su3 = h[1] == 0;
   op.link12 = c->links_su3 ? 1 : 0;
@@ -819,12 +831,14 @@ static int create_impl(wd_ctx* c, const void* links, const int dims[4], cudaStre
     set_err("a 6x6 clover block A_D is singular for kappa=%g c_SW=%g", op.kappa, op.csw);
     return WD_BREAKDOWN;
   }
-  if (op.links_unitary) {   // the fixed-point form of the FP64 stencil (its bounds need unitary links)
-    // one block: an allocation costs as much as building a small lattice's tables
-    const size_t tables = V * ((FX_WSTR + 2 * FX_DSTR + 2) * sizeof(int4) + 3 * WD_LMAX * sizeof(short));
-    c->small_field_bytes = small_field_bytes(V);
-    CU(cudaMalloc(&op.fx_links, tables + c->small_field_bytes));
-    c->small_field = reinterpret_cast<char*>(op.fx_links) + tables;
+  if (!op.links_unitary) {   // the fixed-point stencil's bounds need unitary links
+    op.fx_links = nullptr;
+  } else {
+    if (!op.fx_links) {
+      CU(cudaMalloc(&c->tables, tables));
+      op.fx_links = static_cast<int4*>(c->tables);
+    }
+    c->small_field = reinterpret_cast<char*>(op.fx_links) + V * FX_SITE_BYTES;
     op.fx_clov = op.fx_links + V * FX_WSTR;
     op.fx_cinv = op.fx_clov + V * FX_DSTR;
     op.fx_nb = op.fx_cinv + V * FX_DSTR;
