@@ -835,7 +835,12 @@ static int create_impl(wd_ctx* c, const void* links, const int dims[4], cudaStre
     op.fx_links = nullptr;
   } else {
     if (!op.fx_links) {
-      CU(cudaMalloc(&c->tables, tables));
+      // no room: every product on the FP64 pipe, as links that are not unitary have it
+      if (cudaMalloc(&c->tables, tables) != cudaSuccess) {
+        cudaGetLastError();
+        c->tables = nullptr;
+        return WD_OK;
+      }
       op.fx_links = static_cast<int4*>(c->tables);
     }
     c->small_field = reinterpret_cast<char*>(op.fx_links) + V * FX_SITE_BYTES;
@@ -999,7 +1004,8 @@ int wd_set_apply_form(wd_ctx* c, int form) {
   if (!c) { set_err("ctx is NULL"); return WD_EINVAL; }
   if (form != 0 && form != 1) { set_err("stencil form %d not in {0, 1}", form); return WD_EINVAL; }
   if (form == 1 && !c->op.fx_links) {
-    set_err("the fixed-point stencil needs links whose rows and columns have norm <= 1 + %g", LINK12_TOL);
+    if (c->op.links_unitary) set_err("there was no device memory for the fixed-point stencil's tables");
+    else set_err("the fixed-point stencil needs links whose rows and columns have norm <= 1 + %g", LINK12_TOL);
     return WD_EINVAL;
   }
   c->op.apply_form = form;
