@@ -342,10 +342,14 @@ typedef struct {
   /* Halo exchange on host buffers of `bytes` each: send_lo is this rank's first interior slice
    * (the previous rank's upper halo), send_hi its last interior slice (the next rank's lower
    * halo); recv_lo receives the previous rank's last interior slice, recv_hi the next rank's
-   * first (periodic in t). */
+   * first (periodic in t).  A slice is N x L complex128 as above, or, between the FP64 Jacobi sweeps when
+   * every rank has wd_get_apply_form 1 (the ranks sum a flag through `allreduce` at each call that sweeps),
+   * the same number of bytes in the library's fixed-point form followed by one 2-byte exponent per (site,
+   * right-hand side) and zeros: to be moved as bytes.  `bytes` is a multiple of 16 and the buffers are
+   * 16-byte aligned. */
   int (*exchange)(const void* send_lo, const void* send_hi, void* recv_lo, void* recv_hi,
                   size_t bytes, void* user);
-  /* Sum of n doubles over all ranks, in place in the host buffer `buf`; every rank must get the
+  /* Sum of n doubles (n >= 1) over all ranks, in place in the host buffer `buf`; every rank must get the
    * same result. */
   int (*allreduce)(double* buf, int n, void* user);
   void* user;

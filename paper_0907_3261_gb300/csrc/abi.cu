@@ -152,6 +152,7 @@ struct wd_ctx {
   // each side; halo exchanges and sums over ranks go through the caller's callbacks
   bool dom_on = false;
   wd_domain dom{};
+  bool dom_fields = false;         // this call's FP64 sweeps exchange iterates in fixed point (all ranks do)
   void* dom_host = nullptr;        // pinned staging: 4 halo slices, then the reduction buffer
   size_t dom_host_bytes = 0;
 };
@@ -436,9 +437,13 @@ long long slice_sites(const wd_ctx* c) {
   return (long long)c->op.g.d[0] * c->op.g.d[1] * c->op.g.d[2];
 }
 constexpr int DOM_REDUCE_DOUBLES = 2 * WD_LMAX * WD_LMAX + 2 * WD_LMAX;
+// A halo slice's exponents, padded so that the slices that a callback gets stay 16-byte aligned.
+size_t exponent_bytes(const wd_ctx* c, int L) {
+  return ((size_t)slice_sites(c) * L * sizeof(short) + 15) / 16 * 16;
+}
 
 int dom_staging(wd_ctx* c, int L) {
-  const size_t slice = (size_t)slice_sites(c) * L * (12 * 16 + sizeof(short)) + 16;
+  const size_t slice = (size_t)slice_sites(c) * L * 12 * 16 + exponent_bytes(c, L);
   const size_t need = 4 * slice + DOM_REDUCE_DOUBLES * sizeof(double);
   if (c->dom_host_bytes >= need) return WD_OK;
   if (c->dom_host) cudaFreeHost(c->dom_host);
@@ -457,14 +462,16 @@ int halo_exchange(wd_ctx* c, void* blk, int L, cudaStream_t s, short* exps = nul
   CHECK(dom_staging(c, L));
   const long long Vs = slice_sites(c), V = c->op.g.V;
   const size_t site = (size_t)12 * L * 16, esite = (size_t)L * sizeof(short);   // bytes per site
-  const size_t body = (size_t)Vs * site, slice = body + (exps ? Vs * esite : 0);
+  const size_t body = (size_t)Vs * site, pad = exps ? exponent_bytes(c, L) : 0, slice = body + pad;
   char* h = static_cast<char*>(c->dom_host);
   char* d = static_cast<char*>(blk);
   char* e = reinterpret_cast<char*>(exps);
   const long long from[2] = {Vs, V - 2 * Vs}, to[2] = {0, V - Vs};
   for (int k = 0; k < 2; ++k) {
     CU(cudaMemcpyAsync(h + k * slice, d + from[k] * site, body, cudaMemcpyDeviceToHost, s));
-    if (e) CU(cudaMemcpyAsync(h + k * slice + body, e + from[k] * esite, Vs * esite, cudaMemcpyDeviceToHost, s));
+    if (!e) continue;
+    std::memset(h + k * slice + body + Vs * esite, 0, pad - Vs * esite);
+    CU(cudaMemcpyAsync(h + k * slice + body, e + from[k] * esite, Vs * esite, cudaMemcpyDeviceToHost, s));
   }
   CU(cudaStreamSynchronize(s));
   if (c->dom.exchange(h, h + slice, h + 2 * slice, h + 3 * slice, slice, c->dom.user) != 0) {
@@ -475,6 +482,23 @@ int halo_exchange(wd_ctx* c, void* blk, int L, cudaStream_t s, short* exps = nul
     CU(cudaMemcpyAsync(d + to[k] * site, h + (2 + k) * slice, body, cudaMemcpyHostToDevice, s));
     if (e) CU(cudaMemcpyAsync(e + to[k] * esite, h + (2 + k) * slice + body, Vs * esite, cudaMemcpyHostToDevice, s));
   }
+  return WD_OK;
+}
+
+// Whether the FP64 sweeps' iterates are fields on every rank: the halo slices are in one form, so a rank
+// whose links do not allow the fixed-point one, or that was set to form 0, takes the others along.
+int dom_agree_on_fields(wd_ctx* c, cudaStream_t s) {
+  c->dom_fields = c->op.apply_form == 1;
+  if (!c->dom_on) return WD_OK;
+  CHECK(dom_staging(c, 1));
+  double* h = static_cast<double*>(c->dom_host);
+  *h = c->dom_fields ? 0.0 : 1.0;
+  CU(cudaStreamSynchronize(s));
+  if (c->dom.allreduce(h, 1, c->dom.user) != 0) {
+    set_err("wd_domain.allreduce failed");
+    return WD_ECUDA;
+  }
+  c->dom_fields = *h == 0.0;
   return WD_OK;
 }
 
@@ -572,7 +596,8 @@ int precondition(wd_ctx* c, const double* R, double* a, double* b, double** res,
   }
   double* cur = a;
   double* nxt = b;
-  const bool fields = op.apply_form == 1 && j >= 2;    // the iterates in fixed point up to the last sweep
+  // the iterates in fixed point up to the last sweep
+  const bool fields = op.apply_form == 1 && j >= 2 && (!c->dom_on || c->dom_fields);
   if (fields)
     LAUNCH(WD_K_SITE_INV, 1, launch_first_fx(op, R, a, 0, L, s));
   else
@@ -1095,6 +1120,7 @@ int jacobi_precond(wd_ctx* c, const void* R, void* G, int L, int j, int precisio
   double* first = (j % 2 == 1) ? gd : tmp;
   double* second = (j % 2 == 1) ? tmp : gd;
   if (precision != PM_F64) { first = gd; second = tmp; }   // low-precision sweeps finish in `first`
+  if (j >= 2) CHECK(dom_agree_on_fields(c, s));
   CHECK(precondition(c, rd, first, second, &res, L, j, precision, nullptr, s));
   if (res != gd) LAUNCH(WD_K_COPY, 0, cudaMemcpyAsync(gd, res, bytes, cudaMemcpyDeviceToDevice, s));
   if (!g_dev) CU(cudaMemcpyAsync(G, gd, bytes, cudaMemcpyDeviceToHost, s));
@@ -1237,6 +1263,7 @@ int bbicggr_solve(wd_ctx* c, const void* B, void* X, int L, int j, double tol,
   double b2[WD_LMAX];
   LAUNCH(WD_K_COLNORM, 2, launch_colnorms(Bd + off, L, rows, static_cast<double2*>(c->part.p), c->bnorm2_dev, s));
   CHECK(dom_sum(c, c->bnorm2_dev, L, s));
+  if (j >= 2) CHECK(dom_agree_on_fields(c, s));
   CU(cudaMemcpyAsync(b2, c->bnorm2_dev, L * sizeof(double), cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
   for (int i = 0; i < L; ++i)
