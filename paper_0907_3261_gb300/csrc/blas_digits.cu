@@ -13,24 +13,27 @@
 // through shared memory.
 //
 // Scales: in block times matrix, a power of two per row of the block, per row and per column of the
-// matrix (its entries are first divided by their row's scale, which goes to the block's column, so a block
-// with columns of very different size loses nothing).  In a Gram product, a power of two per column of
+// matrix (its entries are first divided by their row's scale, which goes to the block's column, so that columns of
+// very different size lose nothing where the matrix makes up for them, as alpha and gamma do).  An element none
+// of whose terms comes within DG_SPAN bits of these scales (a nearly diagonal matrix and a factor that much below
+// the largest of its row) is computed again in FP64, and so are elements with subnormals among their factors.  In a Gram product, a power of two per column of
 // either block, held by a warp from tile to tile while the columns' largest elements stay within 2^-7 of
 // it; the warp's sums are 64-bit integers and go to FP64 when a scale changes or after GR_TILES tiles.
-// An infinity or a NaN makes its row of a product, and its row or column of a Gram product, NaN.
+// An infinity or a NaN makes its row of a product, and its row or column of a Gram product, infinite or NaN.
 //
 // A warp takes 16 rows at a time: thread (g, t) = (lane / 4, lane % 4) holds rows g, g + 8 and columns
 // t + 4 i, i < NI = ceil(L / 4).  That is the layout of an mma A fragment with (re, im) as its pairs, and of
 // the accumulators, so products need no exchange; a Gram product contracts over the rows, and movmatrix
 // transposes the digits of both blocks.  Partial sums are added in a fixed order, bitwise reproducible.
 //
-// Measured on a GB300, 16^3x32, L = 12, with the call's 50 us: U 0.29 ms against 0.62 in FP32 pairs and 1.76
-// on the FP64 pipe; P and V 0.98 against 1.81 and 4.90; X and R 0.69 against 0.95 and 2.66.  L = 1: 0.10,
-// 0.26 and 0.26 ms against 0.10, 0.36 and 0.46 (FP32 pairs); 4^4, L = 4: as before, 35 to 60 us.  Bytes alone
+// Measured on a GB300, 16^3x32, L = 12, with the call's 50 us: U 0.30 ms against 0.62 in FP32 pairs and 1.76
+// on the FP64 pipe; P and V 0.98 against 1.81 and 4.90; X and R 0.69 against 0.95 and 2.66 (looking for elements to
+// be computed again takes 0.01 of U's and P and V's).  L = 1: 0.11,
+// 0.27 and 0.26 ms against 0.10, 0.36 and 0.46 (FP32 pairs); 4^4, L = 4: as before, 35 to 60 us.  Bytes alone
 // would take 0.14, 0.32 and 0.41 ms.  X and R is at 76% of the FP64 pipe (their updates stay FP64); the others
 // are bound by the latency of a tile's chain at 12 to 16 warps per SM (tensor pipe 33 to 44%, integer pipe
 // 35 to 42%).  P and V in three blocks of 168 registers against four of 128 and spills: 0.98 against 1.01 ms
-// (L = 16: 1.38 against 1.57); two copies of the product's code for U and Y, 1.08.  Scales without a bit to
+// (L = 16: 1.59 in three); two copies of the product's code for U and Y, 1.08.  Scales without a bit to
 // spare, more flushes: 1.15 ms.
 #include <type_traits>
 
@@ -47,6 +50,12 @@ constexpr int DG_WARPS = DG_TPB / 32;
 constexpr int GR_TILES = 8;                // |tile sum| <= 2^59.1: 8 of them stay below 2^63
 constexpr int GR_WINDOW = 7;               // bits by which a column may fall below its scale
 constexpr int DG_BAD = 1 << 20;            // an exponent that marks an infinity or a NaN
+// Bits by which the factor of a sum's largest term may fall below its row's scale: the digits then keep 2^-44 of
+// the term (seven) or 2^-54 (eight).  Each bit less takes four times as many elements to be computed again: of a
+// diagonal matrix and Gaussian columns 2.5e-4 at 7 bits, where P and V took 1.07 ms, 1.6e-5 at 9 (0.98).
+template <int ND>
+constexpr int DG_SPAN = ND == 8 ? 7 : 9;
+constexpr int DG_TINY = 64;                // exponent fields up to this one: subnormals beside them count
 constexpr unsigned DG_MAGIC = 0x4B400000u;   // 1.5 2^23
 
 WD_DEV void mma16(float c[4], const unsigned a[4], unsigned b0, unsigned b1) {
@@ -70,6 +79,10 @@ WD_DEV unsigned hfma2(unsigned a, unsigned b, unsigned c) {
   return d;
 }
 WD_DEV int raw_exponent(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
+// v is not zero (v with an exponent field of at most DG_TINY).
+WD_DEV bool nonzero(double2 v) {
+  return ((__double2hiint(v.x) | __double2hiint(v.y)) & 0x7FFFFFFF) | __double2loint(v.x) | __double2loint(v.y);
+}
 
 // |v| >> sh as an integer of 8 ND - 1 bits for a v in [1, 2) 2^e at sh = 0, plus 128 in every byte below the
 // top digit's.  FP64 subnormals count as zero.
@@ -131,73 +144,117 @@ WD_DEV i64 joined(const int j[ND], unsigned b) {
   return (i64)B * (1 << (16 + UP)) + ((i64)C * (1 << UP) + D) + ((i64)A << (32 + UP));
 }
 
+// t + z f
+WD_DEV double2 axpy(double2 t, double2 z, double2 f) {
+  return make_double2(fma(-z.y, f.y, fma(z.x, f.x, t.x)), fma(z.y, f.x, fma(z.x, f.y, t.y)));
+}
+
 // ---------------------------------------------------------------- block times matrix
 // The digits of an L x L matrix as mma B fragments, and its scales.
 template <int NI, int ND>
 struct Coef {
   unsigned d[NI * NI * ND * 32];           // [column tile][entry group][digit][lane]
-  int row[4 * NI], col[4 * NI];            // exponents: |m_ab| < 2^(row + col - 1022)
+  int rmax[4 * NI], cmax[4 * NI];          // largest exponent field of a row; 4096 + of a column less its row's scale
+  unsigned tops[4 * NI];                   // bits a: entry (a, b) has column b's scale; LOST: subnormals
+  int lost;                                // some column has them
+  static constexpr unsigned LOST = 1u << 31;
+  // |m_ab| < 2^(row + col - 1022); a row or column of zeros has any scale
+  WD_DEV int row(int a) const { return rmax[a] ? rmax[a] - 1023 : 0; }
+  WD_DEV int col(int b) const { return cmax[b] == 0 ? 1023 : cmax[b] == DG_BAD ? DG_BAD : cmax[b] - 4096; }
+  // which factors of a row of the block make a term of the column's scale
+  WD_DEV unsigned top(int b) const { return tops[b] & LOST ? 0 : cmax[b] == 0 ? 0xFFFFu : tops[b]; }
 };
 
 // Fills `t` from the matrix m, staged in `st` (L^2 entries); ends with a barrier.
 template <int NI, int ND>
 WD_DEV void load_coef(Coef<NI, ND>& t, double2* st, const double2* __restrict__ m, int L) {
   const int tid = threadIdx.x;
-  if (tid < 4 * NI) t.row[tid] = t.col[tid] = 0;
+  if (tid < 4 * NI) t.rmax[tid] = t.cmax[tid] = t.tops[tid] = 0;
+  if (!tid) t.lost = 0;
   __syncthreads();
   // exponent fields: 0 for zero, 2047 for an infinity or a NaN, which do not count for a row's scale
   for (int e = tid; e < L * L; e += DG_TPB) {
     const double2 v = st[e] = m[e];
     const int x = fx::exponent_of(v);
-    if (x && x < 2047) atomicMax(&t.row[e / L], x);
+    if (x && x < 2047) atomicMax(&t.rmax[e / L], x);
   }
   __syncthreads();
-  if (tid < 4 * NI) t.row[tid] = t.row[tid] ? t.row[tid] - 1023 : 0;
-  __syncthreads();
-  // columns, shifted by 4096 so that zero stands for none
   for (int e = tid; e < L * L; e += DG_TPB) {
     const int x = fx::exponent_of(st[e]), a = e / L;
-    if (x) atomicMax(&t.col[e - a * L], x == 2047 ? DG_BAD : 4096 + x - t.row[a]);
+    if (x) atomicMax(&t.cmax[e - a * L], x == 2047 ? DG_BAD : 4096 + x - t.row(a));
   }
   __syncthreads();
-  if (tid < 4 * NI) t.col[tid] = t.col[tid] == 0 ? 1023 : t.col[tid] == DG_BAD ? DG_BAD : t.col[tid] - 4096;
-  __syncthreads();
+  for (int e = tid; e < L * L; e += DG_TPB) {
+    const int x = fx::exponent_of(st[e]), a = e / L, b = e - a * L;
+    if (x <= DG_TINY) {
+      if (nonzero(st[e])) {
+        atomicOr(&t.tops[b], t.LOST);
+        t.lost = 1;
+      }
+    } else if (4096 + x - t.row(a) == t.cmax[b]) {
+      atomicOr(&t.tops[b], 1u << a);
+    }
+  }
   for (int q = tid; q < NI * NI * 32; q += DG_TPB) {
     const int lane = q & 31, ni = q >> 5, i = ni % NI, nt = ni / NI;
-    const int a = (lane & 3) + 4 * i, b = (lane >> 3) + 4 * nt;
+    const int a = (lane & 3) + 4 * i, b = (lane >> 3) + 4 * nt, ra = t.row(a), cb = t.col(b);
     double2 v = make_double2(0.0, 0.0);
     if (a < L && b < L) v = st[a * L + b];
     // column 2b of the real matrix has (re, -im) in rows 2a, 2a + 1, column 2b + 1 (im, re)
     const double x = (lane & 4) ? v.y : v.x, y = (lane & 4) ? v.x : -v.y;
     unsigned d[ND];
-    digits<ND>(biased_at<ND>(x, -t.row[a], t.col[b]), biased_at<ND>(y, -t.row[a], t.col[b]),
-               __double2hiint(x), __double2hiint(y), d);
+    digits<ND>(biased_at<ND>(x, -ra, cb), biased_at<ND>(y, -ra, cb), __double2hiint(x), __double2hiint(y), d);
 #pragma unroll
     for (int k = 0; k < ND; ++k) t.d[(ni * ND + k) * 32 + lane] = d[k];
   }
   __syncthreads();
 }
 
-// The product of the warp's 16 rows with the matrix: put(h, nt, v) gets element (row g + 8 h, column
-// t + 4 nt).
-template <int NI, int ND, class G, class F>
-WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, const G& get, const F& put) {
+// Element (row of A + zeta V, column of m) in FP64 arithmetic; V may be null.  Rare, and so kept small: fetching
+// cold code costs more than the arithmetic.
+__device__ __noinline__ double2 exact_product(const double2* A, const double2* V, double2 zeta, const double2* m,
+                                              int L) {
+  double2 v = make_double2(0.0, 0.0);
+#pragma unroll 1
+  for (int a = 0; a < L; ++a) {
+    double2 x = A[a];
+    if (V) x = axpy(x, zeta, V[a]);
+    v = axpy(v, x, m[a * L]);
+  }
+  return v;
+}
+
+// The product of the warp's 16 rows with the matrix: put(h, nt, base, v) gets element (row g + 8 h, column
+// t + 4 nt), base from get(h, nt).  `ok`: the thread's elements (bits h * NI + i).  Where the digits hold too
+// few bits of a sum's terms -- none has a factor within DG_SPAN of its row's scale and an entry of its column's --
+// exact(h, nt) gives the element in the end, when the digits' registers are free.
+template <int NI, int ND, class G, class X, class F>
+WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, unsigned ok, const G& get, const X& exact,
+                        const F& put) {
   const int lane = threadIdx.x & 31;
   unsigned a[ND][2][NI];
+  constexpr int ZERO = -4000, LOST = DG_BAD - 100;   // exponents of zeros and of what the digits lose
   int E[2];
+  unsigned within = 0;                     // the thread's factors within DG_SPAN of their row's scale
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    int ra[NI];
-    E[h] = -4000;
+    int ra[NI], ex[NI];
+    E[h] = ZERO;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
-      ra[i] = t.row[(lane & 3) + 4 * i];
+      ra[i] = t.row((lane & 3) + 4 * i);
       const int e = fx::exponent_of(in[h][i]);
-      E[h] = max(E[h], e == 2047 ? DG_BAD : e ? e + ra[i] : -4000);
+      ex[i] = e == 2047 ? DG_BAD : e ? e + ra[i] : ZERO;
+      if (e <= DG_TINY && nonzero(in[h][i])) ex[i] = LOST;
+      E[h] = max(E[h], ex[i]);
     }
     E[h] = max(E[h], __shfl_xor_sync(0xFFFFFFFFu, E[h], 1));
     E[h] = max(E[h], __shfl_xor_sync(0xFFFFFFFFu, E[h], 2));
-    if (E[h] == -4000) E[h] = 1023;        // a row of zeros
+    const int lim = E[h] == LOST ? DG_BAD : E[h] - DG_SPAN<ND>;
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if (ex[i] >= lim) within |= 1u << (h * NI + i);
+    if (E[h] == ZERO) E[h] = 1023;         // a row of zeros
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       const double2 v = in[h][i];
@@ -238,7 +295,7 @@ WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, const G&
           mma8(acc[k1 + k2], a[k1][0][NI - 1], a[k1][1][NI - 1], b0);
       }
     }
-    const int C = t.col[(lane & 3) + 4 * nt];
+    const int C = t.col((lane & 3) + 4 * nt);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       int re[ND], im[ND];
@@ -249,6 +306,20 @@ WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, const G&
       }
       put(h, nt, base[h], scaled2(joined<ND, 3>(re, DG_MAGIC), joined<ND, 3>(im, DG_MAGIC), E[h] + C - 2101));
     }
+  }
+  if (__any_sync(0xFFFFFFFFu, (~within & ok) || t.lost)) {
+    unsigned large = 0;                    // bits a (h = 0) and 16 + a: the row's factors within the span
+#pragma unroll
+    for (int q = 0; q < 2 * NI; ++q)
+      if (within >> q & 1) large |= 1u << ((lane & 3) + (q < NI ? 4 * q : 16 + 4 * (q - NI)));
+    large |= __shfl_xor_sync(0xFFFFFFFFu, large, 1);
+    large |= __shfl_xor_sync(0xFFFFFFFFu, large, 2);
+#pragma unroll 1
+    for (int nt = 0; nt < NI; ++nt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if ((ok >> (h * NI + nt) & 1) && !(large >> 16 * h & t.top((lane & 3) + 4 * nt)))
+          put(h, nt, get(h, nt), exact(h, nt));
   }
 }
 
@@ -450,6 +521,10 @@ struct Place {
     }
   }
   WD_DEV bool ok(int h, int i) const { return row[h] && 4 * i < left; }
+  WD_DEV unsigned mask() const {           // bits h * NI + i of the elements that are ok
+    const unsigned m = (1u << max(0, (left + 3) / 4)) - 1;
+    return (row[0] ? m : 0) | (row[1] ? m << NI : 0);
+  }
   WD_DEV void load(const double* __restrict__ p, double2 v[2][NI]) const {
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -485,11 +560,7 @@ struct Staged {
   }
 };
 WD_DEV double2& at(double* p, size_t e) { return reinterpret_cast<double2*>(p)[e]; }
-WD_DEV double2 at(const double* p, size_t e) { return reinterpret_cast<const double2*>(p)[e]; }
-// t + z f
-WD_DEV double2 axpy(double2 t, double2 z, double2 f) {
-  return make_double2(fma(-z.y, f.y, fma(z.x, f.x, t.x)), fma(z.y, f.x, fma(z.x, f.y, t.y)));
-}
+WD_DEV const double2& at(const double* p, size_t e) { return reinterpret_cast<const double2*>(p)[e]; }
 
 // U = (P - zeta V) alpha
 template <int NI, int ND>
@@ -523,7 +594,11 @@ update_u_dg_kernel(const double* __restrict__ P, const double* __restrict__ V, d
 #pragma unroll
       for (int i = 0; i < NI; ++i) s[h][i] = axpy(s[h][i], mz, v[h][i]);
     row_product<NI, ND>(
-        s, al, [](int, int) { return make_double2(0.0, 0.0); },
+        s, al, pl.mask(), [](int, int) { return make_double2(0.0, 0.0); },
+        [&](int h, int nt) {
+          const size_t r = pl.e[h] - (threadIdx.x & 3);
+          return exact_product(&at(P, r), &at(V, r), mz, st->alpha + (threadIdx.x & 3) + 4 * nt, L);
+        },
         [&](int h, int nt, double2, double2 u) {
           if (pl.ok(h, nt)) at(U, pl.e[h] + 4 * nt) = u;
         });
@@ -641,8 +716,12 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
         pl.load(c ? Y : U, u);
       }
       row_product<NI, ND>(
-          u, ga,
+          u, ga, pl.mask(),
           [&](int h, int nt) { return pl.ok(h, nt) ? at(base, pl.e[h] + 4 * nt) : make_double2(0.0, 0.0); },
+          [&](int h, int nt) {
+            return exact_product(&at(c ? Y : U, pl.e[h] - (threadIdx.x & 3)), nullptr, double2(),
+                                 st->gamma + (threadIdx.x & 3) + 4 * nt, L);
+          },
           [&](int h, int nt, double2 w, double2 p) {
             if (!pl.ok(h, nt)) return;
             const double2 x = make_double2(w.x + p.x, w.y + p.y);
