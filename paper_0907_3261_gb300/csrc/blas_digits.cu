@@ -48,7 +48,8 @@ using fx::u64;
 constexpr int DG_TPB = 128;                // 4 warps
 constexpr int DG_WARPS = DG_TPB / 32;
 constexpr int GR_TILES = 8;                // |tile sum| <= 2^59.1: 8 of them stay below 2^63
-constexpr int GR_WINDOW = 7;               // bits by which a column may fall below its scale
+constexpr int GR_WINDOW = 3;               // bits by which a tile's column may fall below its scale
+constexpr int GR_SPAN = 4;                 // bits by which the factors of a tile's largest product may (GR_WINDOW at least)
 constexpr int DG_BAD = 1 << 20;            // an exponent that marks an infinity or a NaN
 // Bits by which the factor of a sum's largest term may fall below its row's scale: the digits then keep 2^-44 of
 // the term (seven) or 2^-54 (eight).  Each bit less takes four times as many elements to be computed again: of a
@@ -324,6 +325,60 @@ WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, unsigned
 }
 
 // ---------------------------------------------------------------- Gram product
+// The larger part's high word without its sign (its exponent above 20 bits), at least 1 for what is not zero.
+WD_DEV unsigned word(double2 v) {
+  const unsigned x = (__double2hiint(v.x) & 0x7FFFFFFF) | min((unsigned)__double2loint(v.x), 1u);
+  const unsigned y = (__double2hiint(v.y) & 0x7FFFFFFF) | min((unsigned)__double2loint(v.y), 1u);
+  return max(x, y);
+}
+// The least word of an element within GR_SPAN of a scale.
+WD_DEV unsigned span_word(int E) { return (unsigned)max(E - GR_SPAN, DG_TINY + 1) << 20; }
+
+// A tile of `n` rows without one whose elements are all within the span.  A product loses nothing if some row has
+// both factors within it, or if either column is zero; if one does lose, adds A^H B to this thread's elements of
+// `out` in FP64 arithmetic and returns true.  ea, eb: the scales of columns t + 4 i.  Rare (see exact_product).
+__device__ __noinline__ bool add_in_fp64(double2* out, int ld, const double2* A, const double2* B, int n, int L,
+                                         int4 ea, int4 eb) {
+  const int lane = threadIdx.x & 31, g = lane >> 2;
+  bool lossy = false;
+#pragma unroll 1
+  for (int mt = 0; mt < 2; ++mt) {
+    const int e0 = __shfl_sync(0xFFFFFFFFu, mt ? ea.z : ea.x, g >> 1);
+    const int e1 = __shfl_sync(0xFFFFFFFFu, mt ? ea.w : ea.y, g >> 1);
+    const unsigned la = span_word((g & 1) ? e1 : e0);
+    const int a = 8 * mt + 4 * (g & 1) + (g >> 1);
+#pragma unroll 1
+    for (int nt = 0; nt < 4; ++nt) {
+      const unsigned lb = span_word(nt == 0 ? eb.x : nt == 1 ? eb.y : nt == 2 ? eb.z : eb.w);
+      const int b = (lane & 3) + 4 * nt;
+      if (a >= L || b >= L) continue;
+      bool some = false, za = true, zb = true;
+#pragma unroll 4
+      for (int r = 0; r < n; ++r) {
+        const unsigned x = word(A[(size_t)r * L + a]), y = word(B[(size_t)r * L + b]);
+        some = some || (x >= la && y >= lb);
+        za = za && !x;
+        zb = zb && !y;
+      }
+      lossy = lossy || !(some || za || zb);
+    }
+  }
+  if (!__any_sync(0xFFFFFFFFu, lossy)) return false;
+#pragma unroll 1
+  for (int a = 4 * (g & 1) + (g >> 1); a < L; a += 8)
+#pragma unroll 1
+    for (int b = lane & 3; b < L; b += 4) {
+      double2 v = out[a * ld + b];
+#pragma unroll 1
+      for (int r = 0; r < n; ++r) {
+        const double2 x = A[(size_t)r * L + a];
+        v = axpy(v, make_double2(x.x, -x.y), B[(size_t)r * L + b]);
+      }
+      out[a * ld + b] = v;
+    }
+  return true;
+}
+
 // One warp's A^H B: element (a, b), a = 8 mt + 4 (g % 2) + g / 2 and b = t + 4 nt, belongs to thread (g, t).
 template <int NI, int ND>
 struct Gram {
@@ -366,37 +421,65 @@ struct Gram {
     }
     tiles = 0;
   }
-  // Scales for the columns of a tile; true when some column left its window.
-  WD_DEV static int column(const double2 v[2][NI], int i, unsigned& bad, int bit) {
-    int e = max(fx::exponent_of(v[0][i]), fx::exponent_of(v[1][i]));
-    if (e == 2047) {
+  // The largest word of a tile's column from this thread's two; an infinity or a NaN sets `bit` of `bad`.
+  WD_DEV static unsigned column(unsigned w0, unsigned w1, unsigned& bad, int bit) {
+    unsigned w = max(w0, w1);
+    if (w >= 0x7FF00000u) {
       bad |= 1u << bit;
-      e = 2046;
+      w = 0x7FE00000u;
     }
-    e = max(e, __shfl_xor_sync(0xFFFFFFFFu, e, 4));
-    e = max(e, __shfl_xor_sync(0xFFFFFFFFu, e, 8));
-    return max(e, __shfl_xor_sync(0xFFFFFFFFu, e, 16));
+    w = max(w, __shfl_xor_sync(0xFFFFFFFFu, w, 4));
+    w = max(w, __shfl_xor_sync(0xFFFFFFFFu, w, 8));
+    return max(w, __shfl_xor_sync(0xFFFFFFFFu, w, 16));
   }
-  WD_DEV void tile(const double2 A[2][NI], const double2 B[2][NI]) {
+  // A tile of the rows from n0 on.  `pa`, `pb`: the blocks, whose rows the warp may have just written.
+  WD_DEV void tile(const double2 A[2][NI], const double2 B[2][NI], const double* pa, const double* pb, long long n0,
+                   long long n1, int L) {
     {
-      int na[NI], nb[NI];
-      bool moved = tiles == GR_TILES;
+      unsigned wa[2][NI], wb[2][NI], ca[NI], cb[NI];
+      bool moved = tiles == GR_TILES;      // some column left its window
 #pragma unroll
       for (int i = 0; i < NI; ++i) {
-        na[i] = column(A, i, bad, i);
-        nb[i] = column(B, i, bad, 8 + i);
-        moved = moved || na[i] > ea[i] || nb[i] > eb[i] || (na[i] && na[i] < ea[i] - GR_WINDOW) ||
-                (nb[i] && nb[i] < eb[i] - GR_WINDOW);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          wa[h][i] = word(A[h][i]);
+          wb[h][i] = word(B[h][i]);
+        }
+        ca[i] = column(wa[0][i], wa[1][i], bad, i);
+        cb[i] = column(wb[0][i], wb[1][i], bad, 8 + i);
+        const int na = ca[i] >> 20, nb = cb[i] >> 20;
+        moved = moved || na > ea[i] || nb > eb[i] || (na && na < ea[i] - GR_WINDOW) ||
+                (nb && nb < eb[i] - GR_WINDOW);
       }
       if (__any_sync(0xFFFFFFFFu, moved)) {
         if (tiles) flush();
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
-          if (na[i] || ea[i] < 0) ea[i] = na[i] + (ea[i] >= 0);   // from the second time on with a bit to spare
-          if (nb[i] || eb[i] < 0) eb[i] = nb[i] + (eb[i] >= 0);
+          const int na = ca[i] >> 20, nb = cb[i] >> 20;
+          if (na || ea[i] < 0) ea[i] = na + (ea[i] >= 0);   // from the second time on with a bit to spare
+          if (nb || eb[i] < 0) eb[i] = nb + (eb[i] >= 0);
         }
       }
       ++tiles;
+      // A row whose elements are all within the span makes products that are.
+      bool in0 = true, in1 = true;         // this quad's elements of rows g and g + 8 (a column of zeros loses nothing)
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const unsigned la = ca[i] ? span_word(ea[i]) : 0, lb = cb[i] ? span_word(eb[i]) : 0;
+        in0 = in0 && wa[0][i] >= la && wb[0][i] >= lb;
+        in1 = in1 && wa[1][i] >= la && wb[1][i] >= lb;
+      }
+      const unsigned r0 = __ballot_sync(0xFFFFFFFFu, in0), r1 = __ballot_sync(0xFFFFFFFFu, in1);
+      const unsigned p0 = r0 & r0 >> 1, p1 = r1 & r1 >> 1;
+      if (!((p0 & p0 >> 2 | p1 & p1 >> 2) & 0x11111111u)) {
+        auto four = [](const int e[NI]) {
+          return make_int4(e[0], NI > 1 ? e[NI > 1 ? 1 : 0] : 0, NI > 2 ? e[NI > 2 ? 2 : 0] : 0, NI > 3 ? e[NI > 3 ? 3 : 0] : 0);
+        };
+        __syncwarp();                      // the warp may have just written the rows
+        if (add_in_fp64(out, LD, reinterpret_cast<const double2*>(pa) + n0 * L, reinterpret_cast<const double2*>(pb) + n0 * L,
+                        (int)min(16LL, n1 - n0), L, four(ea), four(eb)))
+          return;
+      }
     }
     unsigned b[NI][2][ND];
 #pragma unroll
@@ -630,7 +713,7 @@ gram_dg_kernel(const double* __restrict__ A, const double* __restrict__ B, int L
 #pragma unroll
         for (int i = 0; i < NI; ++i) nacc[i] = fma(b[h][i].x, b[h][i].x, fma(b[h][i].y, b[h][i].y, nacc[i]));
     }
-    gr.tile(a, b);
+    gr.tile(a, b, A, B, q * 16, rows, L);
   }
   gr.write(part, outs[0], nred, L, norms ? nacc : nullptr);
 }
@@ -671,7 +754,7 @@ update_xr_dg_kernel(double* __restrict__ X, const double* __restrict__ F, const 
         nacc[i] = fma(r[h][i].x, r[h][i].x, fma(r[h][i].y, r[h][i].y, nacc[i]));
       }
     pl.load(Rt, rt);
-    gr.tile(rt, r);
+    gr.tile(rt, r, Rt, R, q * 16, rows, L);
   }
   gr.write(part, outs[0], nred, L, nacc);
 }
@@ -737,7 +820,7 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
     } else {
       pl.load(Rt, u);
     }
-    gr.tile(u, v);
+    gr.tile(u, v, Rt, V, q * 16, rows, L);
   }
   gr.write(part, outs[0], nullptr, L, nullptr);
 }

@@ -85,3 +85,31 @@ def test_products(wd, dims, L, spread, precision):
             lim = eps * (np.abs(wide(A, L)) @ ca) + 2.0 ** -52 * np.abs(wide(base, L)) + low
             assert (np.abs(wide(host(got), L) - ref) <= lim).all(), kind
     wd.wd_destroy(ctx)
+
+
+@pytest.mark.parametrize("precision", [1])
+@pytest.mark.parametrize("spread", ["none", "columns", "entries", "points", "where the other is small"])
+@pytest.mark.parametrize("dims,L", [((3, 3, 3, 3), 2), ((2, 3, 2, 5), 4), ((3, 3, 3, 5), 7), ((4, 4, 4, 4), 12),
+                                    ((3, 3, 5, 3), 16)])
+def test_gram_products(wd, dims, L, spread, precision):
+    """R~^H V with V = W (gamma = 0) and R~^H R with R unchanged (zeta = 0, Y = 0).  A tile of 16 rows adds at most
+    2 U a row of the terms' moduli, and its sums are added up a few at a time: 64 U in all."""
+    rng = np.random.default_rng(L)
+    n = 12 * int(np.prod(dims))
+    A, B = blocks("none" if spread[0] == "w" else spread, n, L, rng, 2)
+    if spread[0] == "w":
+        few = rng.random((n, 1)) < 0.02                  # rows of R~ that are not zero, where the other block is small
+        A, B = A * few, B * np.where(few, 1e-13, 1.0)
+        A[::37] *= 1e-290
+        A[5] = 1e-315
+    ctx = context(wd, dims)
+    lim = 64 * (2.0 ** -53 if precision == 0 else 2.0 ** -44) * (np.abs(A).T @ np.abs(B)) + 2.0 ** -1060
+    ref = A.astype(np.clongdouble).conj().T @ B.astype(np.clongdouble)
+    a, b = (dev(x.reshape(-1, 12, L)) for x in (A, B))
+    zero, out = dev(np.zeros((n // 12, 12, L), complex)), dev(np.zeros((n // 12, 12, L), complex))
+    none = np.zeros((L, L), complex)
+    got = wd.bb_update_pv(ctx, out, zero.clone(), b, b, b, b, a, none, precision=precision)
+    assert (np.abs(got - ref) <= lim).all()
+    got, norms = wd.bb_update_xr(ctx, out, zero, zero, b, zero, zero, a, 0.0, precision=precision)
+    assert (np.abs(got - ref) <= lim).all()
+    wd.wd_destroy(ctx)
