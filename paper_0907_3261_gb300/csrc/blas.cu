@@ -315,8 +315,9 @@ int ts_max_blocks() { return max_blocks(); }
 
 cudaError_t launch_gram(const double* A, const double* B, int L, long long rows, double2* part,
                         SolverState* st, int which, bool norms_of_b, cudaStream_t s) {
-  const int nb = digit_blocks(rows, L > 12 ? 3 : 4);
-  launch_gram_dg(A, B, L, rows, nb, part, norms_of_b, s);
+  const int nb = digit_blocks(rows, gram_blocks(L, false));
+  const cudaError_t e = launch_gram_dg(A, B, L, rows, nb, part, norms_of_b, s);
+  if (e != cudaSuccess) return e;
   finalize(part, nb, L, st, which, norms_of_b ? st->rnorm2 : nullptr, false, s);
   return cudaGetLastError();
 }
@@ -349,15 +350,16 @@ cudaError_t launch_solve_gamma(SolverState* st, int L, cudaStream_t s) {
 
 cudaError_t launch_update_u(const double* P, const double* V, double* U, int L, long long rows,
                             const SolverState* st, cudaStream_t s, bool df) {
-  return launch_update_u_dg(P, V, U, L, rows, digit_blocks(rows, 4), st, s, df);
+  return launch_update_u_dg(P, V, U, L, rows, digit_blocks(rows, update_u_blocks(L, df)), st, s, df);
 }
 
 cudaError_t launch_update_xr(double* X, const double* F, const double* G, double* R,
                              const double* W, const double* Y, const double* Rt, int L,
                              long long rows, double2* part, SolverState* st, cudaStream_t s,
                              bool df) {
-  const int nb = digit_blocks(rows, L > 12 ? 3 : 4);
-  launch_update_xr_dg(X, F, G, R, W, Y, Rt, L, rows, nb, part, st, s, df);
+  const int nb = digit_blocks(rows, gram_blocks(L, df));
+  const cudaError_t e = launch_update_xr_dg(X, F, G, R, W, Y, Rt, L, rows, nb, part, st, s, df);
+  if (e != cudaSuccess) return e;
   finalize(part, nb, L, st, GRAM_RTR_NEW, st->rnorm2, false, s);
   return cudaGetLastError();
 }
@@ -366,8 +368,9 @@ cudaError_t launch_update_pv(double* P, double* V, const double* R, const double
                              const double* U, const double* Y, const double* Rt, int L,
                              long long rows, double2* part, SolverState* st, cudaStream_t s,
                              bool df) {
-  const int nb = digit_blocks(rows, L > 8 ? 3 : 4);
-  launch_update_pv_dg(P, V, R, W, U, Y, Rt, L, rows, nb, part, st, s, df);
+  const int nb = digit_blocks(rows, update_pv_blocks(L, df));
+  const cudaError_t e = launch_update_pv_dg(P, V, R, W, U, Y, Rt, L, rows, nb, part, st, s, df);
+  if (e != cudaSuccess) return e;
   finalize(part, nb, L, st, GRAM_RTV, nullptr, false, s);
   return cudaGetLastError();
 }

@@ -13,12 +13,16 @@
 // through shared memory.
 //
 // Scales: in block times matrix, a power of two per row of the block, per row and per column of the
-// matrix (its entries are first divided by their row's scale, which goes to the block's column, so that columns of
-// very different size lose nothing where the matrix makes up for them, as alpha and gamma do).  An element none
-// of whose terms comes within DG_SPAN bits of these scales (a nearly diagonal matrix and a factor that much below
-// the largest of its row) is computed again in FP64, and so are elements with subnormals among their factors.  In a Gram product, a power of two per column of
-// either block, held by a warp from tile to tile while the columns' largest elements stay within 2^-7 of
-// it; the warp's sums are 64-bit integers and go to FP64 when a scale changes or after GR_TILES tiles.
+// matrix (its entries are first divided by their row's scale, which goes to the block's column, so that columns
+// of very different size lose nothing where the matrix makes up for them, as alpha and gamma do).  In a Gram
+// product, a power of two per column of either block, held by a warp from tile to tile while the columns'
+// largest elements stay within 2^-GR_WINDOW of it; the warp's sums are 64-bit integers and go to FP64 when a scale
+// changes or after GR_TILES tiles.
+//
+// What the common scales would lose is computed in FP64: an element of a product none of whose terms comes
+// within DG_SPAN bits of them (a nearly diagonal matrix and a factor that much below the largest of its row), a
+// tile of a Gram product one of whose columns' products has no row near both scales (add_in_fp64), and whatever
+// has subnormals among its factors.  So every element keeps its own accuracy, whatever the others are.
 // An infinity or a NaN makes its row of a product, and its row or column of a Gram product, infinite or NaN.
 //
 // A warp takes 16 rows at a time: thread (g, t) = (lane / 4, lane % 4) holds rows g, g + 8 and columns
@@ -26,15 +30,15 @@
 // the accumulators, so products need no exchange; a Gram product contracts over the rows, and movmatrix
 // transposes the digits of both blocks.  Partial sums are added in a fixed order, bitwise reproducible.
 //
-// Measured on a GB300, 16^3x32, L = 12, with the call's 50 us: U 0.30 ms against 0.62 in FP32 pairs and 1.76
-// on the FP64 pipe; P and V 0.98 against 1.81 and 4.90; X and R 0.69 against 0.95 and 2.66 (looking for elements to
-// be computed again takes 0.01 of U's and P and V's).  L = 1: 0.11,
-// 0.27 and 0.26 ms against 0.10, 0.36 and 0.46 (FP32 pairs); 4^4, L = 4: as before, 35 to 60 us.  Bytes alone
-// would take 0.14, 0.32 and 0.41 ms.  X and R is at 76% of the FP64 pipe (their updates stay FP64); the others
+// Measured on a GB300, 16^3x32, L = 12, with the call's 50 us, seven digits (double-float mode): U 0.30 ms against
+// 0.62 in FP32 pairs; P and V 1.04 against 1.81; X and R 0.73 against 0.95; eight digits (FP64 mode): 0.37, 1.27
+// and 0.81 against 1.76, 4.90 and 2.66 on the FP64 pipe.  L = 1: 0.11, 0.28 and 0.26 ms against 0.10, 0.36 and 0.46
+// (FP32 pairs); 4^4, L = 4: as before, 35 to 60 us.  Looking for what has to be computed in FP64 takes 0.01 of
+// U's time, 0.07 of P and V's and 0.04 of X and R's.  Bytes alone would take 0.14, 0.32 and 0.41 ms.  X and R is
+// bound by the FP64 pipe (its updates stay FP64); the others
 // are bound by the latency of a tile's chain at 12 to 16 warps per SM (tensor pipe 33 to 44%, integer pipe
-// 35 to 42%).  P and V in three blocks of 168 registers against four of 128 and spills: 0.98 against 1.01 ms
-// (L = 16: 1.59 in three); two copies of the product's code for U and Y, 1.08.  Scales without a bit to
-// spare, more flushes: 1.15 ms.
+// 35 to 42% before the looking).  P and V in three blocks of 168 registers; two copies of the product's code for
+// U and Y overflow the instruction cache.  Scales without a bit to spare, more flushes: slower by 0.18 ms.
 #include <type_traits>
 
 #include "fixed.cuh"
@@ -47,6 +51,7 @@ using fx::u64;
 
 constexpr int DG_TPB = 128;                // 4 warps
 constexpr int DG_WARPS = DG_TPB / 32;
+static_assert(DG_WARPS == 4, "Gram::write adds four warps' sums in pairs");
 constexpr int GR_TILES = 8;                // |tile sum| <= 2^59.1: 8 of them stay below 2^63
 constexpr int GR_WINDOW = 3;               // bits by which a tile's column may fall below its scale
 constexpr int GR_SPAN = 4;                 // bits by which the factors of a tile's largest product may (GR_WINDOW at least)
@@ -125,9 +130,10 @@ WD_DEV double scaled(i64 v, int k) {
   return m ? __hiloint2double(h | ((int)(sg) & 0x80000000), (int)q) : 0.0;
 }
 __device__ __noinline__ double scaled_any(i64 v, int k) { return ldexp(scaled(v, 0), k); }
-WD_DEV double2 scaled2(i64 re, i64 im, int k) {
-  if ((unsigned)(k + 1000) < 1900u) return make_double2(scaled(re, k), scaled(im, k));
-  if (k < DG_BAD / 2) return make_double2(scaled_any(re, k), scaled_any(im, k));
+// re 2^(k + kr), im 2^(k + ki) for small kr, ki.
+WD_DEV double2 scaled2(i64 re, i64 im, int k, int kr = 0, int ki = 0) {
+  if ((unsigned)(k + 900) < 1700u) return make_double2(scaled(re, k + kr), scaled(im, k + ki));
+  if (k < DG_BAD / 2) return make_double2(scaled_any(re, k + kr), scaled_any(im, k + ki));
   const double nan = __longlong_as_double(0x7FF8000000000000LL);
   return make_double2(nan, nan);
 }
@@ -143,6 +149,19 @@ WD_DEV i64 joined(const int j[ND], unsigned b) {
   if constexpr (ND == 8) D = (int)((unsigned)(j[6] << 8) + j[7] - 257u * b + (1u << (15 - UP))) >> (16 - UP);
   else D = (int)(j[6] - b + (1u << (7 - UP))) >> (8 - UP);
   return (i64)B * (1 << (16 + UP)) + ((i64)C * (1 << UP) + D) + ((i64)A << (32 + UP));
+}
+// The same for one sum of a product, in the units of UP = 3 times 2^k: with eight digits the sum moves up by
+// its own leading zeros, so that a small one loses nothing in the 64 bits.
+template <int ND>
+WD_DEV i64 product_sum(const int j[ND], unsigned b, int& k) {
+  k = 0;
+  if constexpr (ND == 7) return joined<ND, 3>(j, b);
+  const int A = (int)((unsigned)(j[0] << 8) + j[1] - 257u * b), B = (int)((unsigned)(j[2] << 8) + j[3] - 257u * b);
+  const int C = (int)((unsigned)(j[4] << 8) + j[5] - 257u * b), D = (int)((unsigned)(j[6] << 8) + j[7] - 257u * b);
+  const i64 hi = (i64)A * 65536 + B, lo = (i64)C * 65536 + D;    // below 2^45; hi counts 2^32
+  const int up = min(__clzll((i64)fx::absbits(hi)) - 2, 32);
+  k = 19 - up;
+  return (i64)((u64)hi << up) + fx::shr_s(lo + (i64)((1ull << (32 - up)) >> 1), 32 - up);
 }
 
 // t + z f
@@ -305,7 +324,9 @@ WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, unsigned
         re[o] = __float_as_int(acc[o][2 * h]);
         im[o] = __float_as_int(acc[o][2 * h + 1]);
       }
-      put(h, nt, base[h], scaled2(joined<ND, 3>(re, DG_MAGIC), joined<ND, 3>(im, DG_MAGIC), E[h] + C - 2101));
+      int kr, ki;
+      const i64 sr = product_sum<ND>(re, DG_MAGIC, kr), si = product_sum<ND>(im, DG_MAGIC, ki);
+      put(h, nt, base[h], scaled2(sr, si, E[h] + C - 2101, kr, ki));
     }
   }
   if (__any_sync(0xFFFFFFFFu, (~within & ok) || t.lost)) {
@@ -331,25 +352,25 @@ WD_DEV unsigned word(double2 v) {
   const unsigned y = (__double2hiint(v.y) & 0x7FFFFFFF) | min((unsigned)__double2loint(v.y), 1u);
   return max(x, y);
 }
-// The least word of an element within GR_SPAN of a scale.
-WD_DEV unsigned span_word(int E) { return (unsigned)max(E - GR_SPAN, DG_TINY + 1) << 20; }
+// The least word of an element within `span` of a scale.
+WD_DEV unsigned span_word(int E, int span) { return (unsigned)max(E - span, DG_TINY + 1) << 20; }
 
-// A tile of `n` rows without one whose elements are all within the span.  A product loses nothing if some row has
-// both factors within it, or if either column is zero; if one does lose, adds A^H B to this thread's elements of
+// A tile of `n` rows without one whose elements are all within GR_SPAN.  A product loses nothing if some row has
+// both factors within `span`, or if either column is zero; if one does lose, adds A^H B to this thread's elements of
 // `out` in FP64 arithmetic and returns true.  ea, eb: the scales of columns t + 4 i.  Rare (see exact_product).
 __device__ __noinline__ bool add_in_fp64(double2* out, int ld, const double2* A, const double2* B, int n, int L,
-                                         int4 ea, int4 eb) {
+                                         int4 ea, int4 eb, int span) {
   const int lane = threadIdx.x & 31, g = lane >> 2;
   bool lossy = false;
 #pragma unroll 1
   for (int mt = 0; mt < 2; ++mt) {
     const int e0 = __shfl_sync(0xFFFFFFFFu, mt ? ea.z : ea.x, g >> 1);
     const int e1 = __shfl_sync(0xFFFFFFFFu, mt ? ea.w : ea.y, g >> 1);
-    const unsigned la = span_word((g & 1) ? e1 : e0);
+    const unsigned la = span_word((g & 1) ? e1 : e0, span);
     const int a = 8 * mt + 4 * (g & 1) + (g >> 1);
 #pragma unroll 1
     for (int nt = 0; nt < 4; ++nt) {
-      const unsigned lb = span_word(nt == 0 ? eb.x : nt == 1 ? eb.y : nt == 2 ? eb.z : eb.w);
+      const unsigned lb = span_word(nt == 0 ? eb.x : nt == 1 ? eb.y : nt == 2 ? eb.z : eb.w, span);
       const int b = (lane & 3) + 4 * nt;
       if (a >= L || b >= L) continue;
       bool some = false, za = true, zb = true;
@@ -465,7 +486,7 @@ struct Gram {
       bool in0 = true, in1 = true;         // this quad's elements of rows g and g + 8 (a column of zeros loses nothing)
 #pragma unroll
       for (int i = 0; i < NI; ++i) {
-        const unsigned la = ca[i] ? span_word(ea[i]) : 0, lb = cb[i] ? span_word(eb[i]) : 0;
+        const unsigned la = ca[i] ? span_word(ea[i], GR_SPAN) : 0, lb = cb[i] ? span_word(eb[i], GR_SPAN) : 0;
         in0 = in0 && wa[0][i] >= la && wb[0][i] >= lb;
         in1 = in1 && wa[1][i] >= la && wb[1][i] >= lb;
       }
@@ -477,7 +498,7 @@ struct Gram {
         };
         __syncwarp();                      // the warp may have just written the rows
         if (add_in_fp64(out, LD, reinterpret_cast<const double2*>(pa) + n0 * L, reinterpret_cast<const double2*>(pb) + n0 * L,
-                        (int)min(16LL, n1 - n0), L, four(ea), four(eb)))
+                        (int)min(16LL, n1 - n0), L, four(ea), four(eb), ND == 8 ? 1 : GR_SPAN))
           return;
       }
     }
@@ -569,14 +590,9 @@ struct Gram {
     double2* p = part + (size_t)blockIdx.x * PART_STRIDE;
     for (int e = threadIdx.x; e < L * L; e += DG_TPB) {
       const int a = e / L, b = e - a * L;
-      double2 v = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int k = 0; k < DG_WARPS; ++k) {
-        const double2 x = all[k * LD * LD + a * LD + b];
-        v.x += x.x;
-        v.y += x.y;
-      }
-      p[e] = v;
+      const double2* w = all + a * LD + b;
+      const double2 u = w[0], v = w[LD * LD], x = w[2 * LD * LD], y = w[3 * LD * LD];
+      p[e] = make_double2((u.x + v.x) + (x.x + y.x), (u.y + v.y) + (x.y + y.y));
     }
     if (nacc && threadIdx.x < L) {
       double v = 0.0;
@@ -645,13 +661,25 @@ struct Staged {
 WD_DEV double2& at(double* p, size_t e) { return reinterpret_cast<double2*>(p)[e]; }
 WD_DEV const double2& at(const double* p, size_t e) { return reinterpret_cast<const double2*>(p)[e]; }
 
+// Blocks per SM of the three kinds of kernels; their shared memory beyond 48 KB is dynamic.
+constexpr int u_blocks(int NI, int ND) { return ND == 8 && NI >= 3 ? 3 : 4; }
+constexpr int gram_blocks(int NI, int ND) { return NI == 4 || (ND == 8 && NI == 3) ? 3 : 4; }
+constexpr int pv_blocks(int NI, int) { return NI >= 3 ? 3 : 4; }
+extern __shared__ __align__(16) unsigned char dg_smem[];
+
+template <int NI, int ND>
+struct ShU {
+  Staged<NI> sp, sv;                       // sp is also the matrix's stage
+  Coef<NI, ND> al;
+};
 // U = (P - zeta V) alpha
 template <int NI, int ND>
-__global__ void __launch_bounds__(DG_TPB, 4)
+__global__ void __launch_bounds__(DG_TPB, u_blocks(NI, ND))
 update_u_dg_kernel(const double* __restrict__ P, const double* __restrict__ V, double* __restrict__ U, int L,
                    long long rows, const SolverState* __restrict__ st) {
-  __shared__ Coef<NI, ND> al;
-  __shared__ Staged<NI> sp, sv;            // sp is also the matrix's stage
+  ShU<NI, ND>& sh = *reinterpret_cast<ShU<NI, ND>*>(dg_smem);
+  Staged<NI>&sp = sh.sp, &sv = sh.sv;
+  Coef<NI, ND>& al = sh.al;
   if (st->status != ST_OK) return;
   const double2 z = st->zeta, mz = make_double2(-z.x, -z.y);
   load_coef(al, &sp.slot[0][0], st->alpha, L);
@@ -690,7 +718,7 @@ update_u_dg_kernel(const double* __restrict__ P, const double* __restrict__ V, d
 
 // Partial A^H B, and the column norms of B.
 template <int NI, int ND>
-__global__ void __launch_bounds__(DG_TPB, NI == 4 ? 3 : 4)
+__global__ void __launch_bounds__(DG_TPB, gram_blocks(NI, ND))
 gram_dg_kernel(const double* __restrict__ A, const double* __restrict__ B, int L, long long rows,
                double2* __restrict__ part, bool norms) {
   using Gr = Gram<NI, ND>;
@@ -720,7 +748,7 @@ gram_dg_kernel(const double* __restrict__ A, const double* __restrict__ B, int L
 
 // X += zeta F + G;  R -= zeta W + Y;  partial R~_0^H R_{k+1} and ||r_i||^2.
 template <int NI, int ND>
-__global__ void __launch_bounds__(DG_TPB, NI == 4 ? 3 : 4)
+__global__ void __launch_bounds__(DG_TPB, gram_blocks(NI, ND))
 update_xr_dg_kernel(double* __restrict__ X, const double* __restrict__ F, const double* __restrict__ G,
                     double* __restrict__ R, const double* __restrict__ W, const double* __restrict__ Y,
                     const double* __restrict__ Rt, int L, long long rows, double2* __restrict__ part,
@@ -759,20 +787,29 @@ update_xr_dg_kernel(double* __restrict__ X, const double* __restrict__ F, const 
   gr.write(part, outs[0], nred, L, nacc);
 }
 
+template <int NI, int ND>
+struct ShPv {
+  static constexpr bool ST = NI < 4;       // NI = 4: three blocks per SM would not fit
+  Staged<ST ? NI : 1> sg;
+  i64 sums[Gram<NI, ND>::NV][DG_TPB];      // also the matrix's stage
+  double2 outs[DG_WARPS][16 * NI * NI];
+  Coef<NI, ND> ga;
+};
 // P = R + U gamma;  V = W + Y gamma;  partial R~_0^H V_{k+1}.
 template <int NI, int ND>
-__global__ void __launch_bounds__(DG_TPB, NI >= 3 ? 3 : 4)
+__global__ void __launch_bounds__(DG_TPB, pv_blocks(NI, ND))
 update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double* __restrict__ R,
                     const double* __restrict__ W, const double* __restrict__ U, const double* __restrict__ Y,
                     const double* __restrict__ Rt, int L, long long rows, double2* __restrict__ part,
                     const SolverState* __restrict__ st) {
   using Gr = Gram<NI, ND>;
-  __shared__ Coef<NI, ND> ga;
-  __shared__ __align__(16) i64 sums[Gr::NV][DG_TPB];
-  __shared__ double2 outs[DG_WARPS][Gr::LD * Gr::LD];
-  constexpr bool ST = NI < 4;              // NI = 4: beyond 48 KB of static shared memory
-  __shared__ Staged<ST ? NI : 1> sg_;
-  Staged<NI>& sg = reinterpret_cast<Staged<NI>&>(sg_);
+  using Sh = ShPv<NI, ND>;
+  constexpr bool ST = Sh::ST;
+  Sh& sh = *reinterpret_cast<Sh*>(dg_smem);
+  auto& sums = sh.sums;
+  auto& outs = sh.outs;
+  Coef<NI, ND>& ga = sh.ga;
+  Staged<NI>& sg = reinterpret_cast<Staged<NI>&>(sh.sg);
   if (st->status != ST_OK) return;
   const long long tiles = (rows + 15) / 16, step = (long long)gridDim.x * DG_WARPS;
   const long long q0 = (long long)blockIdx.x * DG_WARPS + (threadIdx.x >> 5);
@@ -825,28 +862,47 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
   gr.write(part, outs[0], nullptr, L, nullptr);
 }
 
-// Calls f with the kernels' NI and ND.  Seven digits have the error of an FP64 sum from L = 4 on: relative to
-// U's rms, rms 1.23e-16 and largest 6.3e-16 at L = 4 (FP64 sums 1.19e-16 and 9.1e-16), 1.56e-16 and 9e-16 at
-// L = 12 on 8^4 (1.79e-16 and 1.6e-15); the shorter sums of FP64 mode take eight (L = 1: 0.79e-16,
-// against 0.93e-16 with seven and 0.83e-16 in FP64).  In the double-float updates seven are 30 times as exact
-// as the FP32 pairs were.
+// Calls f with the kernels' NI and ND.  Seven digits for the double-float updates, of which they are 30 times as
+// exact as the FP32 pairs were, and eight for FP64's: a term is then off by less than 2^-58 of the largest factors'
+// product, and the error that is left is the result's one rounding (relative to U's rms at L = 1 0.79e-16,
+// against 0.93e-16 with seven and 0.83e-16 in FP64; at L = 4 seven had 1.23e-16 against 1.19e-16).
 template <class F>
-cudaError_t with_shape(int L, bool df, const F& f) {
-  using std::integral_constant;
-  if (L < 4 && !df) f(integral_constant<int, 1>(), integral_constant<int, 8>());
-  else if (L <= 4) f(integral_constant<int, 1>(), integral_constant<int, 7>());
-  else if (L <= 8) f(integral_constant<int, 2>(), integral_constant<int, 7>());
-  else if (L <= 12) f(integral_constant<int, 3>(), integral_constant<int, 7>());
-  else f(integral_constant<int, 4>(), integral_constant<int, 7>());
-  return cudaGetLastError();
+auto with_shape(int L, bool df, const F& f) {
+  auto ni = [&](auto nd) {
+    using std::integral_constant;
+    if (L <= 4) return f(integral_constant<int, 1>(), nd);
+    if (L <= 8) return f(integral_constant<int, 2>(), nd);
+    if (L <= 12) return f(integral_constant<int, 3>(), nd);
+    return f(integral_constant<int, 4>(), nd);
+  };
+  return df ? ni(std::integral_constant<int, 7>()) : ni(std::integral_constant<int, 8>());
+}
+template <class K>
+cudaError_t allow_smem(K kernel, size_t bytes) {
+  return bytes <= 48 * 1024 ? cudaSuccess
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 }  // namespace
 
+int update_u_blocks(int L, bool df) {
+  return with_shape(L, df, [](auto ni, auto nd) { return u_blocks(ni(), nd()); });
+}
+int gram_blocks(int L, bool df) {
+  return with_shape(L, df, [](auto ni, auto nd) { return gram_blocks(ni(), nd()); });
+}
+int update_pv_blocks(int L, bool df) {
+  return with_shape(L, df, [](auto ni, auto nd) { return pv_blocks(ni(), nd()); });
+}
+
 cudaError_t launch_update_u_dg(const double* P, const double* V, double* U, int L, long long rows, int nb,
                                const SolverState* st, cudaStream_t s, bool df) {
   return with_shape(L, df, [&](auto ni, auto nd) {
-    update_u_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(P, V, U, L, rows, st);
+    constexpr size_t bytes = sizeof(ShU<ni(), nd()>);
+    const cudaError_t e = allow_smem(update_u_dg_kernel<ni(), nd()>, bytes);
+    if (e != cudaSuccess) return e;
+    update_u_dg_kernel<ni(), nd()><<<nb, DG_TPB, bytes, s>>>(P, V, U, L, rows, st);
+    return cudaGetLastError();
   });
 }
 
@@ -854,6 +910,7 @@ cudaError_t launch_gram_dg(const double* A, const double* B, int L, long long ro
                            bool norms, cudaStream_t s) {
   return with_shape(L, false, [&](auto ni, auto nd) {
     gram_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(A, B, L, rows, part, norms);
+    return cudaGetLastError();
   });
 }
 
@@ -862,6 +919,7 @@ cudaError_t launch_update_xr_dg(double* X, const double* F, const double* G, dou
                                 double2* part, const SolverState* st, cudaStream_t s, bool df) {
   return with_shape(L, df, [&](auto ni, auto nd) {
     update_xr_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(X, F, G, R, W, Y, Rt, L, rows, part, st);
+    return cudaGetLastError();
   });
 }
 
@@ -869,6 +927,10 @@ cudaError_t launch_update_pv_dg(double* P, double* V, const double* R, const dou
                                 const double* Y, const double* Rt, int L, long long rows, int nb,
                                 double2* part, const SolverState* st, cudaStream_t s, bool df) {
   return with_shape(L, df, [&](auto ni, auto nd) {
-    update_pv_dg_kernel<ni(), nd()><<<nb, DG_TPB, 0, s>>>(P, V, R, W, U, Y, Rt, L, rows, part, st);
+    constexpr size_t bytes = sizeof(ShPv<ni(), nd()>);
+    const cudaError_t e = allow_smem(update_pv_dg_kernel<ni(), nd()>, bytes);
+    if (e != cudaSuccess) return e;
+    update_pv_dg_kernel<ni(), nd()><<<nb, DG_TPB, bytes, s>>>(P, V, R, W, U, Y, Rt, L, rows, part, st);
+    return cudaGetLastError();
   });
 }

@@ -158,6 +158,9 @@ enum { GRAM_RTR = 0, GRAM_RTR_NEW = 1, GRAM_RTV = 2 };
 
 // The three updates and the Gram products, products in exact digits on the tensor cores (blas_digits.cu); nb: grid size,
 // at most ts_max_blocks().
+int update_u_blocks(int L, bool df);   // blocks per SM, for nb
+int gram_blocks(int L, bool df);       // (launch_gram_dg, launch_update_xr_dg)
+int update_pv_blocks(int L, bool df);
 cudaError_t launch_update_u_dg(const double* P, const double* V, double* U, int L, long long rows, int nb,
                                const SolverState* st, cudaStream_t s, bool df);
 cudaError_t launch_gram_dg(const double* A, const double* B, int L, long long rows, int nb, double2* part,

@@ -58,7 +58,7 @@ def blocks(kind, n, L, rng, count):
 MATRICES = ["identity", "diagonal", "upper", "lower", "nearly diagonal", "dense", "tiny"]
 
 
-@pytest.mark.parametrize("precision", [1])
+@pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("spread", ["none", "columns", "entries", "points"])
 @pytest.mark.parametrize("dims,L", [((3, 3, 3, 3), 2), ((2, 3, 2, 5), 4), ((3, 3, 3, 5), 7), ((4, 4, 4, 4), 12),
                                     ((3, 3, 5, 3), 16)])
@@ -87,7 +87,7 @@ def test_products(wd, dims, L, spread, precision):
     wd.wd_destroy(ctx)
 
 
-@pytest.mark.parametrize("precision", [1])
+@pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("spread", ["none", "columns", "entries", "points", "where the other is small"])
 @pytest.mark.parametrize("dims,L", [((3, 3, 3, 3), 2), ((2, 3, 2, 5), 4), ((3, 3, 3, 5), 7), ((4, 4, 4, 4), 12),
                                     ((3, 3, 5, 3), 16)])
