@@ -308,14 +308,16 @@ int wd_set_link_reals(wd_ctx* ctx, int reals);
  * preconditioner.  1 (the default for links whose rows and columns have norm <= 1 + 1e-6, so
  * unitary links): 64-bit fixed point on the integer pipes -- spinors as integers of 58 bits with one
  * exponent per (site, right-hand side), the operator as integers of 60 bits, exact sums, one rounding
- * per hop to 2^-58 of the largest entry around the site and one to FP64.  It is more accurate than
- * FP64 arithmetic and over four times as fast on GB300, whose FP64 pipe issues two lanes per clock per
+ * per hop to 2^-58 of the largest entry around the site and one to FP64; where a site's own entries are
+ * far above its neighbours', its site block is applied in FP64 arithmetic, so that small components keep
+ * their accuracy beside large ones.  In the norm of a site and its neighbours it is more accurate than
+ * FP64 arithmetic, and over four times as fast on GB300, whose FP64 pipe issues two lanes per clock per
  * SM.  A product with A copies its operand into a block of this form: small operands (up to 24 MiB) to a
  * place that the context holds from its creation on, a solve's to its workspace, others to a block that the
  * context allocates at the first product with a given L and grows for a larger one (an outgrown block that a
  * captured product uses is kept until wd_destroy).  When there is no room for the block, or while the
  * stream is being captured before the context's first product, the product runs as with 0; a context whose
- * tables of this form (3.6 KB per site) find no room has form 0.  0: every operation on the
+ * tables of this form (3.6 KB per site) find no room has form 0, and |kappa| below 2^-6 runs as form 0.  0: every operation on the
  * FP64 pipe.  Asking for 1 with other links, or without the tables, is WD_EINVAL.  wd_get_apply_form
  * returns the form (-1 for a NULL ctx). */
 int wd_set_apply_form(wd_ctx* ctx, int form);

@@ -286,7 +286,7 @@ size_t small_field_bytes(long long V) {
 // block's address: an outgrown block is then kept until wd_destroy.  (A capture before the first product
 // runs on the FP64 pipe for small operands too: what it computes does not depend on their size.)
 void* field_block(wd_ctx* c, int L, cudaStream_t s) {
-  if (c->op.apply_form != 1) return nullptr;
+  if (!uses_fx(c->op)) return nullptr;
   const size_t bytes = block_bytes(c, L);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   const bool capturing = cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
@@ -488,7 +488,7 @@ int halo_exchange(wd_ctx* c, void* blk, int L, cudaStream_t s, short* exps = nul
 // Whether the FP64 sweeps' iterates are fields on every rank: the halo slices are in one form, so a rank
 // whose links do not allow the fixed-point one, or that was set to form 0, takes the others along.
 int dom_agree_on_fields(wd_ctx* c, cudaStream_t s) {
-  c->dom_fields = c->op.apply_form == 1;
+  c->dom_fields = uses_fx(c->op);
   if (!c->dom_on) return WD_OK;
   CHECK(dom_staging(c, 1));
   double* h = static_cast<double*>(c->dom_host);
@@ -597,7 +597,7 @@ int precondition(wd_ctx* c, const double* R, double* a, double* b, double** res,
   double* cur = a;
   double* nxt = b;
   // the iterates in fixed point up to the last sweep
-  const bool fields = op.apply_form == 1 && j >= 2 && (!c->dom_on || c->dom_fields);
+  const bool fields = uses_fx(op) && j >= 2 && (!c->dom_on || c->dom_fields);
   if (fields)
     LAUNCH(WD_K_SITE_INV, 1, launch_first_fx(op, R, a, 0, L, s));
   else
@@ -671,7 +671,7 @@ int run_bbicggr(wd_ctx* c, const double* B, double* X, int L, int j, int precisi
   double2* part = static_cast<double2*>(c->part.p);
   SolverState* st = c->st;
   // The product's copy of its operand goes to the preconditioner's scratch block, free at every product.
-  auto field = [&]() -> void* { return op.apply_form == 1 ? pT : nullptr; };
+  auto field = [&]() -> void* { return uses_fx(op) ? pT : nullptr; };
   CU(cudaMemsetAsync(&st->status, 0, sizeof(int), s));
 
   // R_0 = B - A X_0;  P_0 = R_0;  R~_0 = R_0
@@ -1307,7 +1307,7 @@ int bbicggr_solve(wd_ctx* c, const void* B, void* X, int L, int j, double tol,
     if (rr.status == RUN_STALLED) rr.status = WD_NOT_CONVERGED;
     // true residual ||b_i - A x_i|| / ||b_i||
     double* T = c->blk[B_T].d();
-    void* const field = c->op.apply_form == 1 ? c->blk[B_W].p : nullptr;   // W is not needed any more
+    void* const field = uses_fx(c->op) ? c->blk[B_W].p : nullptr;   // W is not needed any more
     CHECK(halo_exchange(c, Xd, L, s));
     LAUNCH(WD_K_RESID, stencil_kernels(c->op, field), launch_resid_f64(c->op, Xd, Bd, T, field, L, s));
     ++hops;
@@ -1548,7 +1548,7 @@ int build_run(wd_ctx* c, const JobPtrs& jp, int mode, bool df, bool restore, cud
   SolverState* st = c->st;
   GraphCtl* g = static_cast<GraphCtl*>(c->gctl);
   double* hist = c->ghist;
-  void* const field = op.apply_form == 1 ? T : nullptr;   // free at every product (run_bbicggr)
+  void* const field = uses_fx(op) ? T : nullptr;   // free at every product (run_bbicggr)
 
   cudaGraphConditionalHandle hloop;
   CU(cudaGraphConditionalHandleCreate(&hloop, RB, 0, 0));
@@ -1637,7 +1637,7 @@ int build_job(wd_ctx* c, const JobPtrs& jp, cudaGraph_t G) {
   double2* part = static_cast<double2*>(c->part.p);
   GraphCtl* g = static_cast<GraphCtl*>(c->gctl);
   const bool two_modes = jp.X0 != nullptr;
-  void* const field = op.apply_form == 1 ? c->blk[B_W].p : nullptr;   // W is not needed any more
+  void* const field = uses_fx(op) ? c->blk[B_W].p : nullptr;   // W is not needed any more
 
   cudaGraphConditionalHandle hphase;
   CU(cudaGraphConditionalHandleCreate(&hphase, G, 1, cudaGraphCondAssignDefault));

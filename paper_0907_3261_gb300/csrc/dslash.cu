@@ -207,7 +207,7 @@ inline unsigned grid_for(long long n) { return (unsigned)((n + DS_THREADS - 1) /
 // ------------------------------------------------------------------ launchers (FP64)
 cudaError_t launch_apply_f64(const Op& op, const double* x, double* y, void* field, int L,
                              cudaStream_t st) {
-  if (op.apply_form == 1 && field) return launch_apply_fx(op, x, y, field, L, st);
+  if (uses_fx(op) && field) return launch_apply_fx(op, x, y, field, L, st);
   dslash_kernel<double, double, double, double, MODE_APPLY>
       <<<grid_for((long long)op.g.V * L), DS_THREADS, 0, st>>>(x, y, nullptr, op.links, op.clov,
                                                                op.g, L, op.kappa);
@@ -216,7 +216,7 @@ cudaError_t launch_apply_f64(const Op& op, const double* x, double* y, void* fie
 
 cudaError_t launch_resid_f64(const Op& op, const double* x, const double* b, double* y, void* field,
                              int L, cudaStream_t st) {
-  if (op.apply_form == 1 && field) return launch_resid_fx(op, x, b, y, field, L, st);
+  if (uses_fx(op) && field) return launch_resid_fx(op, x, b, y, field, L, st);
   dslash_kernel<double, double, double, double, MODE_RESID>
       <<<grid_for((long long)op.g.V * L), DS_THREADS, 0, st>>>(x, y, b, op.links, op.clov, op.g,
                                                                L, op.kappa);

@@ -15,6 +15,9 @@
 //     exponent among the eight neighbours and the site itself; each hop's sum is rounded once to
 //     2^-59 of that scale (forward and backward hops with opposite ties, so the roundings have no
 //     bias, which a Jacobi sweep would amplify), and the result is rounded to FP64 once.
+//   * a site whose own spinor is more than 2^FX_APART above all its neighbours' (a point source) has its site
+//     block applied in FP64 arithmetic and only the neighbours aligned: its small components would otherwise be
+//     held to 2^-59 of its largest, where their hopping sums are much finer.
 // Bounds: a field's integers are at most 2^28 in high limbs, so |h| <= 2^29 and |hr +- hi| <= 2^30;
 // link rows have norm <= 1 (checked at creation), so a hop's sums stay below 2^62 and the eight hops'
 // total, in units of 2^FX_UP, below 2^62.3; a block's sum, shifted left by at most FX_CS, and a sweep's
@@ -216,15 +219,32 @@ WD_DEV void store_field(const i64* acc, u64 ob, int eu, bool finite, bool live, 
   if (sp == 0) *ye = (short)(!finite ? FX_NONFINITE : top == -FX_NONFINITE ? FX_EMIN : eu + n);
 }
 
+// Row i of a packed Hermitian block times v in FP64 arithmetic: component j at v[j * step], its imaginary part `im`
+// further on.
+static __device__ __noinline__ double2 row_in_fp64(const double* b, const double* v, int step, int im, int i) {
+  double2 q = make_double2(b[i] * v[i * step], b[i] * v[i * step + im]);
+#pragma unroll 1
+  for (int j = 0; j < 6; ++j) {
+    if (j == i) continue;
+    const int t = i > j ? tri_index(i, j) : tri_index(j, i);
+    const double c = b[t], d = i > j ? b[t + 1] : -b[t + 1], x = v[j * step], y = v[j * step + im];
+    q.x = fma(-d, y, fma(c, x, q.x));
+    q.y = fma(d, x, fma(c, y, q.y));
+  }
+  return q;
+}
+
 // A product with A (APPLY: y = A x, RESID: y = u - A x) or a Jacobi sweep y = A_D^{-1}(u + kappa H x)
-// of the field x (exponents xe); u FP64 (JACOBI: its exponents ue); y FP64, or a field (QOUT).
+// of the field x (exponents xe); u FP64 (JACOBI: its exponents ue); y FP64, or a field (QOUT).  x64 (APPLY, RESID)
+// is x itself, D64 the site blocks: where a site's own spinor is far above its neighbours', the common scale would
+// lose its small components, and the site block is applied in FP64 arithmetic (not for a field, which has one scale).
 // ST: the links and blocks of the CTA's sites are staged in shared memory.
 template <int MODE, bool ST, bool QOUT>
 __global__ void __launch_bounds__(TPB, 4)
 fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __restrict__ y,
           short* __restrict__ ye, const double2* __restrict__ u, const short* __restrict__ ue,
-          const int4* __restrict__ W, const int4* __restrict__ D, const int4* __restrict__ nbt, int V,
-          int L, int ek, int z0) {
+          const double* __restrict__ x64, const double* __restrict__ D64, const int4* __restrict__ W,
+          const int4* __restrict__ D, const int4* __restrict__ nbt, int V, int L, int ek, int z0) {
   const unsigned npair = (unsigned)V * L;            // at most 2^30
   const unsigned p0 = blockIdx.x * (TPB / 2u), p1 = p0 + (threadIdx.x >> 1);
   const bool live = p1 < npair;
@@ -250,7 +270,8 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
   __shared__ i64 acc[2][6][TPB];
   const int t = threadIdx.x;
   const int eo = __ldg((MODE == MODE_JACOBI ? ue : xe) + (size_t)s * L + r);
-  const int E = neighbours_and_scale(nbt, xe + r, s, L, eo, &nbs[0][t]);
+  bool apart;
+  const int E = neighbours_and_scale(nbt, xe + r, s, L, eo, &nbs[0][t], QOUT ? nullptr : &apart);
   const bool finite = E < FX_NONFINITE;
   const char* xo = reinterpret_cast<const char*>(x + (size_t)(3 * sp) * L + r);
   const unsigned stride = 192u * (unsigned)L;        // bytes per site
@@ -290,7 +311,7 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
   const int eh = E + ek - FX_OP + FX_UP;       // the hopping sums' unit: 2^(eh - FX_BIAS)
   Fac v[6];
   if constexpr (MODE != MODE_JACOBI) {
-    const int so = min(E - eo, 60);
+    const int so = apart ? 0 : min(E - eo, 60);
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
       const int4 a = __ldg(x + base + (size_t)i * L);
@@ -308,11 +329,20 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
       block_row<ST>(Dc + 6 * i, v, re, im, z0);
       i64 hr = slot[(2 * i) * TPB], hi = slot[(2 * i + 1) * TPB];
       if (cr) {
-        hr = shr_s(hr, min(cr, 63));
-        hi = shr_s(hi, min(cr, 63));
+        const int c = min(cr, 61);
+        hr = shr_s(hr + (i64)((1ull << c) >> 1), c);
+        hi = shr_s(hi + (i64)((1ull << c) >> 1), c);
       }
       if (!live) continue;
-      double2 q = fx_out((re << cl_) - hr, (im << cl_) - hi, e - FX_BIAS, e, finite);
+      double2 q;
+      if (apart) {
+        q = row_in_fp64(D64 + ((size_t)s * 2 + sp) * CLOV_REALS, x64 + 2 * base, 2 * L, 1, i);
+        const double2 h = fx_out(slot[(2 * i) * TPB], slot[(2 * i + 1) * TPB], eh - FX_BIAS, eh, finite);
+        q.x -= h.x;
+        q.y -= h.y;
+      } else {
+        q = fx_out((re << cl_) - hr, (im << cl_) - hi, e - FX_BIAS, e, finite);
+      }
       if constexpr (MODE == MODE_RESID) {
         const double2 b = __ldg(u + base + (size_t)i * L);
         q.x = b.x - q.x;
@@ -321,6 +351,18 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
       reinterpret_cast<double2*>(y)[base + (size_t)i * L] = q;
     }
   } else {
+    if constexpr (!QOUT) {
+      if (apart) {
+        double* const v64 = reinterpret_cast<double*>(&acc[0][0][t]);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          const double2 a = __ldg(u + base + (size_t)i * L);
+          const double2 h = fx_out(hs[2 * i], hs[2 * i + 1], eh - FX_BIAS, eh, finite);
+          v64[(2 * i) * TPB] = a.x + h.x;
+          v64[(2 * i + 1) * TPB] = a.y + h.y;
+        }
+      }
+    }
     // v = u + kappa H x in the hopping sums' units: |u| = m 2^(ef - 1075), m shifted left by 10
     u64 bits = 0;
 #pragma unroll
@@ -353,7 +395,10 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
         (&acc[0][0][t])[(2 * i) * TPB] = re;
         (&acc[0][0][t])[(2 * i + 1) * TPB] = im;
       } else if (live) {
-        reinterpret_cast<double2*>(y)[base + (size_t)i * L] = fx_out(re, im, eu - FX_BIAS, eu, finite);
+        reinterpret_cast<double2*>(y)[base + (size_t)i * L] =
+            apart ? row_in_fp64(D64 + ((size_t)s * 2 + sp) * CLOV_REALS, reinterpret_cast<double*>(&acc[0][0][t]),
+                                2 * TPB, TPB, i)
+                  : fx_out(re, im, eu - FX_BIAS, eu, finite);
       }
     }
     if constexpr (QOUT)
@@ -534,19 +579,20 @@ constexpr int FX_STAGE_L = 3;
 
 template <int MODE, bool QOUT>
 cudaError_t launch_fx(const Op& op, const int4* x, const short* xe, void* y, short* ye, const double* u,
-                      const short* ue, const int4* D, int L, cudaStream_t st) {
+                      const short* ue, const double* x64, const int4* D, int L, cudaStream_t st) {
   const unsigned grid = grid_of(2LL * op.g.V * L, TPB);
   const double2* u2 = reinterpret_cast<const double2*>(u);
+  const double* D64 = MODE == MODE_JACOBI ? op.clov_inv : op.clov;
   if (L >= FX_STAGE_L) {
     const int bytes = ((TPB / 2 - 1) / L + 2) * (FX_WSTR + FX_DSTR) * (int)sizeof(int4);
     cudaError_t e = cudaFuncSetAttribute(fx_kernel<MODE, true, QOUT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
-    fx_kernel<MODE, true, QOUT><<<grid, TPB, bytes, st>>>(x, xe, y, ye, u2, ue, op.fx_links, D, op.fx_nb,
-                                                          op.g.V, L, op.fx_ek, 0);
+    fx_kernel<MODE, true, QOUT><<<grid, TPB, bytes, st>>>(x, xe, y, ye, u2, ue, x64, D64, op.fx_links, D,
+                                                          op.fx_nb, op.g.V, L, op.fx_ek, 0);
   } else {
-    fx_kernel<MODE, false, QOUT><<<grid, TPB, 0, st>>>(x, xe, y, ye, u2, ue, op.fx_links, D, op.fx_nb,
-                                                       op.g.V, L, op.fx_ek, 0);
+    fx_kernel<MODE, false, QOUT><<<grid, TPB, 0, st>>>(x, xe, y, ye, u2, ue, x64, D64, op.fx_links, D,
+                                                       op.fx_nb, op.g.V, L, op.fx_ek, 0);
   }
   return cudaGetLastError();
 }
@@ -579,14 +625,14 @@ cudaError_t launch_apply_fx(const Op& op, const double* x, double* y, void* q, i
   const cudaError_t e = split(op, x, static_cast<int4*>(q), op.fx_exp(0), L, st);
   if (e != cudaSuccess) return e;
   return launch_fx<MODE_APPLY, false>(op, static_cast<const int4*>(q), op.fx_exp(0), y, nullptr, nullptr,
-                                      nullptr, op.fx_clov, L, st);
+                                      nullptr, x, op.fx_clov, L, st);
 }
 
 cudaError_t launch_resid_fx(const Op& op, const double* x, const double* b, double* y, void* q, int L,
                             cudaStream_t st) {
   const cudaError_t e = split(op, x, static_cast<int4*>(q), op.fx_exp(0), L, st);
   if (e != cudaSuccess) return e;
-  return launch_fx<MODE_RESID, false>(op, static_cast<const int4*>(q), op.fx_exp(0), y, nullptr, b, nullptr,
+  return launch_fx<MODE_RESID, false>(op, static_cast<const int4*>(q), op.fx_exp(0), y, nullptr, b, nullptr, x,
                                       op.fx_clov, L, st);
 }
 
@@ -602,7 +648,7 @@ cudaError_t launch_sweep_fx(const Op& op, const void* q_in, int slot, const doub
   const int4* x = static_cast<const int4*>(q_in);
   if (q_out)
     return launch_fx<MODE_JACOBI, true>(op, x, op.fx_exp(slot), q_out, op.fx_exp(1 - slot), u, op.fx_exp(2),
-                                        op.fx_cinv, L, st);
-  return launch_fx<MODE_JACOBI, false>(op, x, op.fx_exp(slot), g64, nullptr, u, op.fx_exp(2), op.fx_cinv, L,
-                                       st);
+                                        nullptr, op.fx_cinv, L, st);
+  return launch_fx<MODE_JACOBI, false>(op, x, op.fx_exp(slot), g64, nullptr, u, op.fx_exp(2), nullptr,
+                                       op.fx_cinv, L, st);
 }

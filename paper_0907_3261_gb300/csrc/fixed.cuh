@@ -1,4 +1,4 @@
-// Shared by the fixed-point stencils (dslash_fx.cu, sweep_fx.cu): 64-bit integer helpers, conversions
+// The parts of the fixed-point stencil (dslash_fx.cu) that do not depend on its limbs: 64-bit integer helpers, conversions
 // from and to FP64, and the loads of a hop's spinors.  A field is 16 bytes per complex number, site-major
 // [site][spin*3+colour][rhs], with one exponent per (site, rhs); two threads of a warp share one
 // (site, rhs), thread sp the upper spin sp in the hops and chirality sp in the site blocks.
@@ -14,6 +14,7 @@ typedef unsigned long long u64;
 constexpr int FX_EMIN = 1;                 // smallest exponent of a field made from FP64
 constexpr int FX_NONFINITE = 30000;        // the exponent of a spinor with an infinity or a NaN
 constexpr int FX_EK = -4;                  // smallest exponent of the links' scale
+constexpr int FX_APART = 1;                // bits by which a site's field may exceed its neighbours' before its block is done in FP64
 constexpr int TPB = 128;
 constexpr unsigned NB_MASK = (1u << 26) - 1u;
 
@@ -87,18 +88,21 @@ WD_DEV double2 fx_out(i64 re, i64 im, int k, int e, bool finite) {
 WD_DEV u64 absbits(i64 v) { return (u64)(v ^ (v >> 63)); }
 WD_DEV int bit_len(u64 b) { return 64 - __clzll((i64)b); }
 
-// The neighbours of a site with the shifts that align their fields to E, the largest of their exponents
-// and e0, into nbs (one slot of TPB apart per direction; xe points at this right-hand side).
+// The neighbours of a site with the shifts that align their fields to E, into nbs (one slot of TPB apart per
+// direction; xe points at this right-hand side).  E is the largest of their exponents and e0, the site's own, unless
+// `apart` finds e0 more than FX_APART above theirs: then the largest of theirs alone.
 WD_DEV int neighbours_and_scale(const int4* __restrict__ nbt, const short* __restrict__ xe, int s, int L,
-                                int e0, unsigned* nbs) {
+                                int e0, unsigned* nbs, bool* apart) {
   const int4 n0 = __ldg(nbt + 2 * (size_t)s), n1 = __ldg(nbt + 2 * (size_t)s + 1);
   const int nn[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-  int e[8], E = e0;
+  int e[8], E = 0;
 #pragma unroll
   for (int d = 0; d < 8; ++d) {
     e[d] = __ldg(xe + (size_t)nn[d] * L);
     E = max(E, e[d]);
   }
+  if (apart) *apart = e0 > E + FX_APART && e0 < FX_NONFINITE;
+  if (!apart || !*apart) E = max(E, e0);
 #pragma unroll
   for (int d = 0; d < 8; ++d) nbs[d * TPB] = (unsigned)nn[d] | ((unsigned)min(E - e[d], 60) << 26);
   return E;

@@ -49,6 +49,10 @@ struct Op {
   int apply_form;
   short* fx_exp(int slot) const { return fx_exps + (size_t)slot * g.V * WD_LMAX; }
 };
+// Whether the FP64 stencils run in fixed point.  Fields are aligned to the largest of a site and its neighbours,
+// whatever kappa, and are held to 2^-59 of it: at |kappa| >= 2^-6 that stays below what an FP64 sum of the
+// neighbours' part rounds (2^-53 |kappa| of them, several times).  Smaller ones take the FP64 pipe.
+inline bool uses_fx(const Op& op) { return op.apply_form == 1 && (op.kappa >= 0x1p-6 || op.kappa <= -0x1p-6); }
 constexpr int FX_WSTR = 72;   // int4 per site of fx_links
 constexpr int FX_DSTR = 73;   // int4 per site of fx_clov, fx_cinv
 
@@ -81,7 +85,7 @@ cudaError_t launch_first_fx(const Op& op, const double* u, void* q_out, int slot
 cudaError_t launch_sweep_fx(const Op& op, const void* q_in, int slot, const double* u, void* q_out,
                             double* g64, int L, cudaStream_t st);
 // Kernels one FP64 product with A takes (the fixed-point form copies its operand first).
-inline int stencil_kernels(const Op& op, const void* field) { return op.apply_form == 1 && field ? 2 : 1; }
+inline int stencil_kernels(const Op& op, const void* field) { return uses_fx(op) && field ? 2 : 1; }
 
 // ---- sweep_lp.cu, sweep_f32.cu, sweep_bf16.cu: the low-precision preconditioner.  Its private
 // blocks (u_lp, g_lp) are component-major, [spin*3+colour][site][rhs], one complex number per

@@ -99,7 +99,7 @@ extern "C" int jacobi_precond_noalloc(wd_ctx* ctx, const void* R, void* G, int L
     // j sweeps alternate between two blocks; start in G when j is odd so the last lands in G.
     double* cur = (j % 2 == 1) ? g : scratch;
     double* nxt = (j % 2 == 1) ? scratch : g;
-    const bool fields = op.apply_form == 1 && j >= 2;   // the iterates in fixed point, as jacobi_precond
+    const bool fields = uses_fx(op) && j >= 2;   // the iterates in fixed point, as jacobi_precond
     e = fields ? launch_first_fx(op, r, cur, 0, L, s) : launch_site_inverse_f64(op, r, cur, L, s);
     wd_ctx_count_launches(ctx, WD_K_SITE_INV, 1);
     for (int i = 1; i < j && e == cudaSuccess; ++i) {
