@@ -156,6 +156,16 @@ struct Lu {
   double2 extra;                           // a number that the block's last warp computes beside
 };
 
+// conj(c) / n for n = |c|^2.  Where 1 / n would leave the normal range (block norms around 1e-77) the parts are
+// divided one by one; else one reciprocal serves both.
+WD_DEV double2 reciprocal(double2 c, double n) {
+  if (n > 0x1p-1000 && n < 0x1p1000) {
+    const double r = 1.0 / n;
+    return make_double2(c.x * r, -c.y * r);
+  }
+  return make_double2(c.x / n, -c.y / n);
+}
+
 inline int lu_threads(int L) { return (2 * L * L + 31) / 32 * 32 + 32; }
 
 // m: this thread's element (i, j).  On return `order` is row i's place and, for j >= L, m the solution's element
@@ -183,13 +193,13 @@ __device__ bool lu_solve(Lu& s, Cx<double>& m, int L, int i, int j, bool live, i
       s.u[k][j] = d2(m);
     }
     if (live && j == k) {
-      const double pn = __longlong_as_double(best), r = 1.0 / pn;
-      const Cx<double> rp = cmake(s.c[p].x * r, -s.c[p].y * r);
+      const double pn = __longlong_as_double(best);
+      const double2 rp = reciprocal(s.c[p], pn);
       if (mine) {
-        s.rp[k] = d2(rp);
+        s.rp[k] = rp;
         s.pn[k] = pn;
       }
-      s.f[i] = d2(cmul(m, rp));            // the factor of row i (of no use in the pivot's)
+      s.f[i] = d2(cmul(m, sm(rp)));            // the factor of row i (of no use in the pivot's)
     }
     __syncthreads();
     if (live && order == L && j > k) {
@@ -258,8 +268,7 @@ __global__ void solve_gamma_kernel(SolverState* st, int L) {
   const bool live = j < 2 * L;
   if (e == blockDim.x - 32) {
     const double2 z = st->zeta;
-    const double r = 1.0 / (z.x * z.x + z.y * z.y);
-    s.extra = make_double2(z.x * r, -z.y * r);
+    s.extra = reciprocal(z, z.x * z.x + z.y * z.y);
   }
   Cx<double> m = czero<double>();
   if (live) m = j < L ? sm(st->rtr[i * L + j]) : sm(st->rtr_new[i * L + j - L]);

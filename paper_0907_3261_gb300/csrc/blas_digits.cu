@@ -51,7 +51,7 @@ using fx::u64;
 
 constexpr int DG_TPB = 128;                // 4 warps
 constexpr int DG_WARPS = DG_TPB / 32;
-static_assert(DG_WARPS == 4, "Gram::write adds four warps' sums in pairs");
+static_assert(DG_WARPS == 4, "Gram::write adds four warps' sums");
 constexpr int GR_TILES = 8;                // |tile sum| <= 2^59.1: 8 of them stay below 2^63
 constexpr int GR_WINDOW = 3;               // bits by which a tile's column may fall below its scale
 constexpr int GR_SPAN = 4;                 // bits by which the factors of a tile's largest product may (GR_WINDOW at least)
@@ -592,7 +592,7 @@ struct Gram {
       const int a = e / L, b = e - a * L;
       const double2* w = all + a * LD + b;
       const double2 u = w[0], v = w[LD * LD], x = w[2 * LD * LD], y = w[3 * LD * LD];
-      p[e] = make_double2((u.x + v.x) + (x.x + y.x), (u.y + v.y) + (x.y + y.y));
+      p[e] = make_double2(((u.x + v.x) + x.x) + y.x, ((u.y + v.y) + x.y) + y.y);
     }
     if (nacc && threadIdx.x < L) {
       double v = 0.0;
