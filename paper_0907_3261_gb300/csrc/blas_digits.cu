@@ -142,22 +142,22 @@ WD_DEV double2 scaled2(i64 re, i64 im, int k, int kr = 0, int ki = 0) {
 // units of 2^(40 + UP); the orders 6 and 7 are rounded (a floor's bias would grow with the rows of a Gram
 // product).
 template <int ND, int UP>
-WD_DEV i64 joined(const int j[ND], unsigned b) {
-  const int A = (int)((unsigned)(j[0] << 8) + j[1] - 257u * b), B = (int)((unsigned)(j[2] << 8) + j[3] - 257u * b);
-  const int C = (int)((unsigned)(j[4] << 8) + j[5] - 257u * b);
+WD_DEV i64 joined(const unsigned j[ND], unsigned b) {
+  const int A = (int)((j[0] << 8) + j[1] - 257u * b), B = (int)((j[2] << 8) + j[3] - 257u * b);
+  const int C = (int)((j[4] << 8) + j[5] - 257u * b);
   int D;
-  if constexpr (ND == 8) D = (int)((unsigned)(j[6] << 8) + j[7] - 257u * b + (1u << (15 - UP))) >> (16 - UP);
+  if constexpr (ND == 8) D = (int)((j[6] << 8) + j[7] - 257u * b + (1u << (15 - UP))) >> (16 - UP);
   else D = (int)(j[6] - b + (1u << (7 - UP))) >> (8 - UP);
-  return (i64)B * (1 << (16 + UP)) + ((i64)C * (1 << UP) + D) + ((i64)A << (32 + UP));
+  return (i64)B * (1 << (16 + UP)) + ((i64)C * (1 << UP) + D) + (i64)((u64)(i64)A << (32 + UP));
 }
 // The same for one sum of a product, in the units of UP = 3 times 2^k: with eight digits the sum moves up by
 // its own leading zeros, so that a small one loses nothing in the 64 bits.
 template <int ND>
-WD_DEV i64 product_sum(const int j[ND], unsigned b, int& k) {
+WD_DEV i64 product_sum(const unsigned j[ND], unsigned b, int& k) {
   k = 0;
   if constexpr (ND == 7) return joined<ND, 3>(j, b);
-  const int A = (int)((unsigned)(j[0] << 8) + j[1] - 257u * b), B = (int)((unsigned)(j[2] << 8) + j[3] - 257u * b);
-  const int C = (int)((unsigned)(j[4] << 8) + j[5] - 257u * b), D = (int)((unsigned)(j[6] << 8) + j[7] - 257u * b);
+  const int A = (int)((j[0] << 8) + j[1] - 257u * b), B = (int)((j[2] << 8) + j[3] - 257u * b);
+  const int C = (int)((j[4] << 8) + j[5] - 257u * b), D = (int)((j[6] << 8) + j[7] - 257u * b);
   const i64 hi = (i64)A * 65536 + B, lo = (i64)C * 65536 + D;    // below 2^45; hi counts 2^32
   const int up = min(__clzll((i64)fx::absbits(hi)) - 2, 32);
   k = 19 - up;
@@ -318,11 +318,11 @@ WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, unsigned
     const int C = t.col((lane & 3) + 4 * nt);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      int re[ND], im[ND];
+      unsigned re[ND], im[ND];
 #pragma unroll
       for (int o = 0; o < ND; ++o) {
-        re[o] = __float_as_int(acc[o][2 * h]);
-        im[o] = __float_as_int(acc[o][2 * h + 1]);
+        re[o] = __float_as_uint(acc[o][2 * h]);
+        im[o] = __float_as_uint(acc[o][2 * h + 1]);
       }
       int kr, ki;
       const i64 sr = product_sum<ND>(re, DG_MAGIC, kr), si = product_sum<ND>(im, DG_MAGIC, ki);
@@ -548,11 +548,11 @@ struct Gram {
         for (int k2 = 0; k2 < ND; ++k2)
 #pragma unroll
           for (int k1 = 0; k1 + k2 < ND; ++k1) mma16(acc[k1 + k2], a[k1], b[nt][0][k2], b[nt][1][k2]);
-        int re[ND], im[ND];
+        unsigned re[ND], im[ND];
 #pragma unroll
         for (int o = 0; o < ND; ++o) {
-          re[o] = __float_as_int(acc[o][0]) + __float_as_int(acc[o][3]);
-          im[o] = __float_as_int(acc[o][1]) - __float_as_int(acc[o][2]);
+          re[o] = __float_as_uint(acc[o][0]) + __float_as_uint(acc[o][3]);
+          im[o] = __float_as_uint(acc[o][1]) - __float_as_uint(acc[o][2]);
         }
         i64* s = sum + (mt * NI + nt) * 2 * DG_TPB;
         s[0] += joined<ND, 0>(re, 2u * DG_MAGIC);

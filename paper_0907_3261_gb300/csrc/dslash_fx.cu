@@ -124,8 +124,8 @@ WD_DEV void cmadd3(Sum K[3], const Ent& a, const Fac& f) {
 // The two parts plus c; the mixed sums enter in units of 4 of the high ones (2^32 / 2^FX_S), rounded.
 WD_DEV void csum(const Sum K[3], i64 c, int z, i64& re, i64& im) {
   const int m1 = (int)(K[0].m >> 32), m2 = (int)(K[1].m >> 32), m3 = (int)(K[2].m >> 32);
-  re = K[0].h - K[2].h + ((i64)(m1 - m3 + z) << 2) + c;
-  im = K[0].h + K[1].h + ((i64)(m1 + m2 + z) << 2) + c;
+  re = K[0].h - K[2].h + shl((i64)(m1 - m3 + z), 2) + c;
+  im = K[0].h + K[1].h + shl((i64)(m1 + m2 + z), 2) + c;
 }
 
 // Operator tables are read from shared memory (staged) or through the read-only cache.
@@ -315,7 +315,7 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
       const int4 a = __ldg(x + base + (size_t)i * L);
-      v[i] = fac_of(lim_of(((i64)a.x << FX_S) + a.y, FX_S + so), lim_of(((i64)a.z << FX_S) + a.w, FX_S + so), z0);
+      v[i] = fac_of(lim_of(shl(a.x, FX_S) + a.y, FX_S + so), lim_of(shl(a.z, FX_S) + a.w, FX_S + so), z0);
     }
     // the site block's unit is 2^cs of the hopping sums'; with a large block these are shifted instead
     const int cs = eD - ek - FX_UP, cl_ = min(cs, FX_CS), cr = cs - cl_;
@@ -341,7 +341,7 @@ fx_kernel(const int4* __restrict__ x, const short* __restrict__ xe, void* __rest
         q.x -= h.x;
         q.y -= h.y;
       } else {
-        q = fx_out((re << cl_) - hr, (im << cl_) - hi, e - FX_BIAS, e, finite);
+        q = fx_out(shl(re, cl_) - hr, shl(im, cl_) - hi, e - FX_BIAS, e, finite);
       }
       if constexpr (MODE == MODE_RESID) {
         const double2 b = __ldg(u + base + (size_t)i * L);
@@ -501,7 +501,7 @@ WD_DEV Lim limbs_kappa(double v, double kappa, int sc) {
   const u64 mk = mantissa(__double2hiint(kappa), (unsigned)__double2loint(kappa), ek);
   const u64 hi = __umul64hi(m << 11, mk << 11);          // |kappa v| = hi 2^(42 + ef + ek - 2150)
   const Lim a = hi ? signed_limbs(hi, 2150 - 42 - ef - ek - sc, v) : Lim{0, 0};
-  return __double2hiint(kappa) < 0 ? lim_of(-(((i64)a.h << FX_S) + a.l), FX_S) : a;
+  return __double2hiint(kappa) < 0 ? lim_of(-(shl(a.h, FX_S) + a.l), FX_S) : a;
 }
 
 // kappa W for the eight directions of every site (W = U_mu(s) forward, U_mu(s - mu)^H backward), row by

@@ -28,6 +28,7 @@ WD_DEV i64 shr_s(i64 v, int n) {
   asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
   return r;
 }
+WD_DEV i64 shl(i64 v, int n) { return (i64)((u64)v << n); }   // defined for negative v
 WD_DEV void mac(i64& a, int x, int y) { a += (i64)x * y; }
 
 // The magnitude of an FP64 number (words h, l) as a 53-bit integer and a power of two: m 2^(ef - 1075).
