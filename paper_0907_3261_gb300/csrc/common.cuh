@@ -102,13 +102,9 @@ __host__ __device__ constexpr int tri_index(int i, int j) { return 6 + 2 * (i * 
 struct DF {
   float hi, lo;
 };
-WD_DEV DF df_from(double d) {
-  const float hi = __double2float_rn(d);
-  return {hi, __double2float_rn(d - (double)hi)};
-}
 WD_DEV double df_to(DF a) { return (double)a.hi + (double)a.lo; }
-// The same two conversions built from the IEEE-754 bit fields on the integer and FP32 pipes.  On
-// GB300 the FP64 pipe issues two lanes per clock per SM, and the FP64 <-> FP32 conversions above
+// Conversions from and to FP64 built from the IEEE-754 bit fields on the integer and FP32 pipes.  On
+// GB300 the FP64 pipe issues two lanes per clock per SM, and its FP64 <-> FP32 conversions
 // run on it; the bulk conversions of whole blocks use these instead.
 //   df_split: hi = d truncated to 24 significant bits; lo = d - hi rounded to nearest FP32.  The
 //   remainder (29 fraction bits r) enters as two exact differences 2^E (1 + f) - 2^E, one for the
@@ -177,7 +173,6 @@ struct CDF {
   DF re, im;
 };
 WD_DEV Cx<double> cdf_to(CDF z) { return {df_to(z.re), df_to(z.im)}; }
-WD_DEV CDF cdf_split(Cx<double> z) { return {df_split(z.re), df_split(z.im)}; }
 WD_DEV Cx<double> cdf_join(CDF z) { return {df_join(z.re), df_join(z.im)}; }
 WD_DEV CDF cdf_zero() { return {{0.f, 0.f}, {0.f, 0.f}}; }
 // acc += a * b (complex)
