@@ -789,8 +789,7 @@ update_xr_dg_kernel(double* __restrict__ X, const double* __restrict__ F, const 
 
 template <int NI, int ND>
 struct ShPv {
-  static constexpr bool ST = NI < 4;       // NI = 4: three blocks per SM would not fit
-  Staged<ST ? NI : 1> sg;
+  Staged<NI> sg;
   i64 sums[Gram<NI, ND>::NV][DG_TPB];      // also the matrix's stage
   double2 outs[DG_WARPS][16 * NI * NI];
   Coef<NI, ND> ga;
@@ -804,17 +803,15 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
                     const SolverState* __restrict__ st) {
   using Gr = Gram<NI, ND>;
   using Sh = ShPv<NI, ND>;
-  constexpr bool ST = Sh::ST;
   Sh& sh = *reinterpret_cast<Sh*>(dg_smem);
   auto& sums = sh.sums;
   auto& outs = sh.outs;
   Coef<NI, ND>& ga = sh.ga;
-  Staged<NI>& sg = reinterpret_cast<Staged<NI>&>(sh.sg);
+  Staged<NI>& sg = sh.sg;
   if (st->status != ST_OK) return;
   const long long tiles = (rows + 15) / 16, step = (long long)gridDim.x * DG_WARPS;
   const long long q0 = (long long)blockIdx.x * DG_WARPS + (threadIdx.x >> 5);
-  if constexpr (ST)
-    if (q0 < tiles) sg.ask(Place<NI>(q0, L, rows), U);
+  if (q0 < tiles) sg.ask(Place<NI>(q0, L, rows), U);
   load_coef(ga, reinterpret_cast<double2*>(sums), st->gamma, L);
   Gr gr;
   gr.init(&sums[0][threadIdx.x], outs[threadIdx.x >> 5]);
@@ -829,12 +826,8 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
     for (int c = 0; c < 2; ++c) {
       const double* base = c ? W : R;
       double* out = c ? V : P;
-      if constexpr (ST) {
-        sg.take(u);
-        sg.ask(pl, c ? Rt : Y);
-      } else {
-        pl.load(c ? Y : U, u);
-      }
+      sg.take(u);
+      sg.ask(pl, c ? Rt : Y);
       row_product<NI, ND>(
           u, ga, pl.mask(),
           [&](int h, int nt) { return pl.ok(h, nt) ? at(base, pl.e[h] + 4 * nt) : make_double2(0.0, 0.0); },
@@ -851,12 +844,8 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
               if (i == nt) v[h][i] = x;    // V's in the end
           });
     }
-    if constexpr (ST) {
-      sg.take(u);
-      if (q + step < tiles) sg.ask(Place<NI>(q + step, L, rows), U);
-    } else {
-      pl.load(Rt, u);
-    }
+    sg.take(u);
+    if (q + step < tiles) sg.ask(Place<NI>(q + step, L, rows), U);
     gr.tile(u, v, Rt, V, q * 16, rows, L);
   }
   gr.write(part, outs[0], nullptr, L, nullptr);
