@@ -50,7 +50,7 @@ PRECISIONS = {"fp64": 0, "mixed": 1, "bf16": 3, "df": 4, "df_dirs": 5}   # bbicg
 FORM_NAMES = {"fp64": "plain FP64 Jacobi", "mixed": "mixed: FP32 Jacobi preconditioner",
               "bf16": "mixed: Jacobi preconditioner on BF16-stored blocks",
               "df": "mixed: double-float Jacobi preconditioner (FP32 pairs, FP32 operator)",
-              "df_dirs": "mixed: double-float preconditioner and direction recurrences"}
+              "df_dirs": "mixed: double-float preconditioner, direction recurrences in seven digits"}
 # FP32 lane operations (a packed FP32x2 instruction is two) per site and RHS of one double-float
 # sweep, counting a split product (FP32 operator entry x FP32-pair value, added into a sum with
 # two-sum) as 11, the first product of a sum as 3 and a two-sum addition as 8.  Each of the 8 hops: 12 additions for the projection, the link
@@ -74,7 +74,8 @@ DF_OPS_GRID = 8 * (12 * 8 + 6 * (2 * 2 * 14 + 8) + 16 + 24 * 8) + 8 * 30 \
 # hops make 2 spins x 9 of them, the two 6x6 site blocks 72.
 FX_MULS = 9 * (8 * 18 + 72)
 # FP64-pipe and FP32-lane operations per site and RHS of the same stencils with the hopping sums in
-# exact FP32 grid sums (the form before the fixed-point one, kept for comparisons): the spin projections (8 hops x 12 real FMAs), joining
+# exact FP32 grid sums, the form before the fixed-point one (for comparisons with its timings; nothing here
+# runs it): the spin projections (8 hops x 12 real FMAs), joining
 # the three levels of the 24 hopping sums (2 adds each), the 24 final FMAs with kappa, and the two
 # Hermitian 6x6 site blocks (6 real x complex products and 15 complex entries used twice, 4 FMAs per
 # complex product: 2 x (12 + 120)).  The hopping products themselves run on the FP32 lanes: 288

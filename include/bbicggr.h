@@ -27,7 +27,8 @@
  * Ownership: the caller owns every buffer it passes; the library never frees or keeps a pointer to
  * one after the call returns.  wd_create copies the links and derives the clover term into
  * context-owned device memory; solver workspace is allocated at the first call with a given L and
- * kept in the context until wd_destroy.
+ * kept in the context until a solver call with another L or wd_destroy (the operand's copy of wd_apply: see
+ * wd_set_apply_form).
  * Streams: `stream` is a cudaStream_t (NULL = legacy default stream).  All device work of a call is
  * ordered on it.  A context must not be used from two host threads at once.
  * Errors: every entry point returns an int status (WD_OK = 0) and never aborts; wd_strerror gives
@@ -68,14 +69,15 @@ typedef struct {
                              accumulation -- the outer recurrences, the products W = AF and
                              Y = AG, the Gram matrices, the L x L solves and the true residual stay
                              FP64; 2: as 1, and the direction recurrences U = (P - zeta V) alpha,
-                             P = R + U gamma, V = W + Y gamma and the Gram products in double-float
-                             (FP32-pair, ~48-bit) arithmetic on the FP32 pipes, with the X and R
-                             updates and column norms still FP64; 3: as 1 with the
+                             P = R + U gamma, V = W + Y gamma and the Gram products in the accuracy
+                             of double-float (FP32-pair, ~48-bit) arithmetic or better -- seven
+                             base-256 digits, where the other modes take eight -- with the
+                             X and R updates and column norms still FP64; 3: as 1 with the
                              preconditioner's blocks (its copy of U and the sweep iterates) stored
                              in BF16, arithmetic FP32; 4: double-float sweeps -- the operator
                              (links, A_D^{-1}, kappa) in FP32 and the spinors as FP32 pairs
                              (~48 bits), so M is linear to ~1e-13; 5: as 4, and the direction
-                             recurrences in double-float as in 2.  In 1-5 the sweeps read 12-real
+                             recurrences in seven digits as in 2.  In 1-5 the sweeps read 12-real
                              links (rows 0 and 1, row 2 rebuilt) when wd_link_reals says 12 */
   double* history;        /* optional host array: max_i ||r_i||/||b_i|| after every R update */
   int history_len;        /* capacity of history (entries beyond it are dropped) */
@@ -163,10 +165,12 @@ int bbicggr_solve(wd_ctx* ctx, const void* B, void* X, int L, int j, double tol,
  * buffers are WD_EINVAL).  They are the updates bbicggr_solve runs, exposed for tests and for
  * drivers that run the iteration themselves.  L x L matrices are host arrays of L*L complex128,
  * row-major (entry (a, b) at a*L + b); zeta is a host complex128 (re, im).  precision: 0 = FP64;
- * 1 = the products with the L x L matrix and the Gram products in double-float arithmetic (the
+ * 1 = the products with the L x L matrix and the Gram products in double-float accuracy (the
  * direction recurrences of bbicggr_opts.precision 2 and 5); the X and R updates and the column
- * norms are FP64 in both.  Each call synchronises the stream.  Output blocks must not overlap the
- * inputs (X and R are updated in place in bb_update_xr).
+ * norms are FP64 in both.  The products run in exact base-256 digits, eight or (precision 1) seven, and in
+ * FP64 arithmetic where the digits' common scales would cost an element its own accuracy.  Each call
+ * synchronises the stream.  Output blocks must not overlap the inputs (X and R are updated in place in
+ * bb_update_xr).
  *   bb_update_u:  U = (P - zeta V) alpha                         (S_k and U_k of the box)
  *   bb_update_xr: X <- X + zeta F + G,  R <- R - zeta W - Y,  rtr_new = R~_0^H R (new R),
  *                 rnorm2[i] = ||r_i||^2 (new R); rtr_new and rnorm2 may be NULL

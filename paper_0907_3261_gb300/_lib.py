@@ -268,8 +268,8 @@ def bbicggr_solve(ctx: Context, B, X=None, j: int = 12, tol: float = 1e-12, maxi
 
     ``X`` (if given) holds X_0 and receives the solution; by default X_0 = 0.  ``precision``
     picks the preconditioner's arithmetic: 0 FP64 sweeps, 1 FP32 sweeps, 2 as 1 with the direction
-    recurrences in double-float, 3 FP32 arithmetic on BF16 blocks, 4 double-float sweeps, 5 as 4
-    with double-float direction recurrences; in 1-5 a stalled run starts over from X_0 with FP64
+    recurrences in double-float accuracy (seven digits), 3 FP32 arithmetic on BF16 blocks, 4 double-float
+    sweeps, 5 as 4 with the direction recurrences of 2; in 1-5 a stalled run starts over from X_0 with FP64
     sweeps (``info["fallbacks"]``).  Solver outcomes (WD_NOT_CONVERGED, WD_DIVERGED, WD_BREAKDOWN)
     are reported in ``info["status"]``; argument and CUDA errors raise WDError."""
     pb, L, kb = _ptr_and_L(B, "B")
@@ -315,7 +315,7 @@ def _host_c128(a, shape, what):
 
 
 def bb_update_u(ctx: Context, P, V, U, zeta: complex, alpha, precision: int = 0, stream=None):
-    """U = (P - zeta V) alpha on device blocks (precision 1: double-float products)."""
+    """U = (P - zeta V) alpha on device blocks (precision 1: products in double-float accuracy)."""
     pp, L, k1 = _ptr_and_L(P, "P")
     pv, _, k2 = _ptr_and_L(V, "V")
     pu, _, k3 = _ptr_and_L(U, "U")

@@ -10,7 +10,8 @@
 // bits are then the sum as an integer; what is dropped is below 2^-8ND of the largest product.  mma.sync and
 // not tcgen05: a tile is 16 rows by at most 32 columns, and the thread that loads an element also
 // owns the element of the same place in the product, so nothing but the digits of alpha and gamma passes
-// through shared memory.
+// through shared memory.  (Exact products of split factors on matrix units: K. Ozaki, T. Ogita, S. Oishi and
+// S. M. Rump, Numer. Algorithms 59 (2012) 95.)
 //
 // Scales: in block times matrix, a power of two per row of the block, per row and per column of the
 // matrix (its entries are first divided by their row's scale, which goes to the block's column, so that columns

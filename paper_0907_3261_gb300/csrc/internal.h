@@ -60,7 +60,7 @@ constexpr int FX_DSTR = 73;   // int4 per site of fx_clov, fx_cinv
 constexpr double LINK12_TOL = 1e-6;
 
 // ---- dslash.cu (FP64).  `field` is a block for the fixed-point form's copy of x; without one, or
-// with apply_form 0, the product runs on the FP64 pipe.
+// where uses_fx() says no, the product runs on the FP64 pipe.
 cudaError_t launch_apply_f64(const Op& op, const double* x, double* y, void* field, int L,
                              cudaStream_t st);
 cudaError_t launch_resid_f64(const Op& op, const double* x, const double* b, double* y, void* field,
@@ -183,7 +183,7 @@ cudaError_t launch_traces(const double* W, const double* R, int L, long long row
                           double2* part, SolverState* st, cudaStream_t s);
 cudaError_t launch_solve_alpha(SolverState* st, int L, cudaStream_t s);
 cudaError_t launch_solve_gamma(SolverState* st, int L, cudaStream_t s);
-// df: the products with L x L matrices and the Gram products in double-float arithmetic.
+// df: the products with L x L matrices and the Gram products in double-float accuracy (seven digits).
 cudaError_t launch_update_u(const double* P, const double* V, double* U, int L, long long rows,
                             const SolverState* st, cudaStream_t s, bool df);
 cudaError_t launch_update_xr(double* X, const double* F, const double* G, double* R,
