@@ -52,7 +52,7 @@ using fx::u64;
 
 constexpr int DG_TPB = 128;                // 4 warps
 constexpr int DG_WARPS = DG_TPB / 32;
-static_assert(DG_WARPS == 4, "Gram::write adds four warps' sums");
+static_assert(DG_WARPS == 4, "Gram::write adds four warps' sums in pairs");
 constexpr int GR_TILES = 8;                // |tile sum| <= 2^59.1: 8 of them stay below 2^63
 constexpr int GR_WINDOW = 3;               // bits by which a tile's column may fall below its scale
 constexpr int GR_SPAN = 4;                 // bits by which the factors of a tile's largest product may (GR_WINDOW at least)
@@ -231,24 +231,39 @@ WD_DEV void load_coef(Coef<NI, ND>& t, double2* st, const double2* __restrict__ 
   __syncthreads();
 }
 
-// Element (row of A + zeta V, column of m) in FP64 arithmetic; V may be null.  Rare, and so kept small: fetching
+// This lane's element (row of A + zeta V, column t of the four columns at m) in FP64 arithmetic; V may be null.
+// `who`: the lanes that ask.  Each row's four lanes share the sum over the factors.  Rare, and so kept small: fetching
 // cold code costs more than the arithmetic.
 __device__ __noinline__ double2 exact_product(const double2* A, const double2* V, double2 zeta, const double2* m,
-                                              int L) {
-  double2 v = make_double2(0.0, 0.0);
+                                              int L, unsigned who) {
+  const int t = threadIdx.x & 3;
+  double2 mine = make_double2(0.0, 0.0);
 #pragma unroll 1
-  for (int a = 0; a < L; ++a) {
-    double2 x = A[a];
-    if (V) x = axpy(x, zeta, V[a]);
-    v = axpy(v, x, m[a * L]);
+  for (int c = 0; c < 4; ++c) {
+    if (!(who & 0x11111111u << c)) continue;
+    double2 v = make_double2(0.0, 0.0);
+    if (who >> (threadIdx.x & 28) >> c & 1) {
+#pragma unroll 1
+      for (int a = t; a < L; a += 4) {
+        double2 x = A[a];
+        if (V) x = axpy(x, zeta, V[a]);
+        v = axpy(v, x, m[a * L + c]);
+      }
+    }
+#pragma unroll 1
+    for (int k = 1; k < 4; k <<= 1) {
+      v.x += __shfl_xor_sync(0xFFFFFFFFu, v.x, k);
+      v.y += __shfl_xor_sync(0xFFFFFFFFu, v.y, k);
+    }
+    if (t == c) mine = v;
   }
-  return v;
+  return mine;
 }
 
 // The product of the warp's 16 rows with the matrix: put(h, nt, base, v) gets element (row g + 8 h, column
 // t + 4 nt), base from get(h, nt).  `ok`: the thread's elements (bits h * NI + i).  Where the digits hold too
 // few bits of a sum's terms -- none has a factor within DG_SPAN of its row's scale and an entry of its column's --
-// exact(h, nt) gives the element in the end, when the digits' registers are free.
+// exact(h, nt, who) gives it in the end, when the digits' registers are free (who: the lanes that ask).
 template <int NI, int ND, class G, class X, class F>
 WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, unsigned ok, const G& get, const X& exact,
                         const F& put) {
@@ -340,9 +355,14 @@ WD_DEV void row_product(const double2 in[2][NI], const Coef<NI, ND>& t, unsigned
 #pragma unroll 1
     for (int nt = 0; nt < NI; ++nt)
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if ((ok >> (h * NI + nt) & 1) && !(large >> 16 * h & t.top((lane & 3) + 4 * nt)))
-          put(h, nt, get(h, nt), exact(h, nt));
+      for (int h = 0; h < 2; ++h) {
+        const bool lossy = (ok >> (h * NI + nt) & 1) && !(large >> 16 * h & t.top((lane & 3) + 4 * nt));
+        const unsigned who = __ballot_sync(0xFFFFFFFFu, lossy);
+        if (who) {
+          const double2 v = exact(h, nt, who);
+          if (lossy) put(h, nt, get(h, nt), v);
+        }
+      }
   }
 }
 
@@ -357,47 +377,61 @@ WD_DEV unsigned word(double2 v) {
 WD_DEV unsigned span_word(int E, int span) { return (unsigned)max(E - span, DG_TINY + 1) << 20; }
 
 // A tile of `n` rows without one whose elements are all within GR_SPAN.  A product loses nothing if some row has
-// both factors within `span`, or if either column is zero; if one does lose, adds A^H B to this thread's elements of
+// both factors within `span`, or if no row has both; if one does lose, adds A^H B to this thread's elements of
 // `out` in FP64 arithmetic and returns true.  ea, eb: the scales of columns t + 4 i.  Rare (see exact_product).
 __device__ __noinline__ bool add_in_fp64(double2* out, int ld, const double2* A, const double2* B, int n, int L,
                                          int4 ea, int4 eb, int span) {
-  const int lane = threadIdx.x & 31, g = lane >> 2;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // Of this quad's columns (of A, << 16: of B): the rows within the span, the rows that are not zero.
+  unsigned within[4], some[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int c = t + 4 * i;
+    const unsigned la = span_word(i == 0 ? ea.x : i == 1 ? ea.y : i == 2 ? ea.z : ea.w, span);
+    const unsigned lb = span_word(i == 0 ? eb.x : i == 1 ? eb.y : i == 2 ? eb.z : eb.w, span);
+    within[i] = some[i] = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = g + 8 * h;
+      if (c >= L || r >= n) continue;
+      const unsigned x = word(A[(size_t)r * L + c]), y = word(B[(size_t)r * L + c]);
+      within[i] |= (x >= la ? 1u << r : 0) | (y >= lb ? 65536u << r : 0);
+      some[i] |= (x ? 1u << r : 0) | (y ? 65536u << r : 0);
+    }
+#pragma unroll
+    for (int k = 4; k < 32; k <<= 1) {
+      within[i] |= __shfl_xor_sync(0xFFFFFFFFu, within[i], k);
+      some[i] |= __shfl_xor_sync(0xFFFFFFFFu, some[i], k);
+    }
+  }
+  unsigned short rows[8];                  // of this thread's products: the rows with both factors
   bool lossy = false;
-#pragma unroll 1
+#pragma unroll
   for (int mt = 0; mt < 2; ++mt) {
-    const int e0 = __shfl_sync(0xFFFFFFFFu, mt ? ea.z : ea.x, g >> 1);
-    const int e1 = __shfl_sync(0xFFFFFFFFu, mt ? ea.w : ea.y, g >> 1);
-    const unsigned la = span_word((g & 1) ? e1 : e0, span);
-    const int a = 8 * mt + 4 * (g & 1) + (g >> 1);
-#pragma unroll 1
+    const unsigned w0 = __shfl_sync(0xFFFFFFFFu, within[2 * mt], g >> 1), w1 = __shfl_sync(0xFFFFFFFFu, within[2 * mt + 1], g >> 1);
+    const unsigned s0 = __shfl_sync(0xFFFFFFFFu, some[2 * mt], g >> 1), s1 = __shfl_sync(0xFFFFFFFFu, some[2 * mt + 1], g >> 1);
+    const unsigned w = (g & 1) ? w1 : w0, s = (g & 1) ? s1 : s0;
+#pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-      const unsigned lb = span_word(nt == 0 ? eb.x : nt == 1 ? eb.y : nt == 2 ? eb.z : eb.w, span);
-      const int b = (lane & 3) + 4 * nt;
-      if (a >= L || b >= L) continue;
-      bool some = false, za = true, zb = true;
-#pragma unroll 4
-      for (int r = 0; r < n; ++r) {
-        const unsigned x = word(A[(size_t)r * L + a]), y = word(B[(size_t)r * L + b]);
-        some = some || (x >= la && y >= lb);
-        za = za && !x;
-        zb = zb && !y;
-      }
-      lossy = lossy || !(some || za || zb);
+      const unsigned both = s & some[nt] >> 16;
+      rows[4 * mt + nt] = (unsigned short)both;
+      lossy = lossy || ((both & 0xFFFFu) && !(w & within[nt] >> 16));
     }
   }
   if (!__any_sync(0xFFFFFFFFu, lossy)) return false;
 #pragma unroll 1
-  for (int a = 4 * (g & 1) + (g >> 1); a < L; a += 8)
+  for (int q = 0; q < 8; ++q) {
+    const int a = 8 * (q >> 2) + 4 * (g & 1) + (g >> 1), b = t + 4 * (q & 3);
+    if (!rows[q]) continue;                // also columns beyond L
+    double2 v = out[a * ld + b];
 #pragma unroll 1
-    for (int b = lane & 3; b < L; b += 4) {
-      double2 v = out[a * ld + b];
-#pragma unroll 1
-      for (int r = 0; r < n; ++r) {
-        const double2 x = A[(size_t)r * L + a];
-        v = axpy(v, make_double2(x.x, -x.y), B[(size_t)r * L + b]);
-      }
-      out[a * ld + b] = v;
+    for (unsigned m = rows[q]; m; m &= m - 1) {
+      const size_t r = (size_t)(__ffs((int)m) - 1) * L;
+      const double2 x = A[r + a];
+      v = axpy(v, make_double2(x.x, -x.y), B[r + b]);
     }
+    out[a * ld + b] = v;
+  }
   return true;
 }
 
@@ -593,7 +627,7 @@ struct Gram {
       const int a = e / L, b = e - a * L;
       const double2* w = all + a * LD + b;
       const double2 u = w[0], v = w[LD * LD], x = w[2 * LD * LD], y = w[3 * LD * LD];
-      p[e] = make_double2(((u.x + v.x) + x.x) + y.x, ((u.y + v.y) + x.y) + y.y);
+      p[e] = make_double2((u.x + v.x) + (x.x + y.x), (u.y + v.y) + (x.y + y.y));
     }
     if (nacc && threadIdx.x < L) {
       double v = 0.0;
@@ -707,9 +741,9 @@ update_u_dg_kernel(const double* __restrict__ P, const double* __restrict__ V, d
       for (int i = 0; i < NI; ++i) s[h][i] = axpy(s[h][i], mz, v[h][i]);
     row_product<NI, ND>(
         s, al, pl.mask(), [](int, int) { return make_double2(0.0, 0.0); },
-        [&](int h, int nt) {
+        [&](int h, int nt, unsigned who) {
           const size_t r = pl.e[h] - (threadIdx.x & 3);
-          return exact_product(&at(P, r), &at(V, r), mz, st->alpha + (threadIdx.x & 3) + 4 * nt, L);
+          return exact_product(&at(P, r), &at(V, r), mz, st->alpha + 4 * nt, L, who);
         },
         [&](int h, int nt, double2, double2 u) {
           if (pl.ok(h, nt)) at(U, pl.e[h] + 4 * nt) = u;
@@ -832,9 +866,9 @@ update_pv_dg_kernel(double* __restrict__ P, double* __restrict__ V, const double
       row_product<NI, ND>(
           u, ga, pl.mask(),
           [&](int h, int nt) { return pl.ok(h, nt) ? at(base, pl.e[h] + 4 * nt) : make_double2(0.0, 0.0); },
-          [&](int h, int nt) {
-            return exact_product(&at(c ? Y : U, pl.e[h] - (threadIdx.x & 3)), nullptr, double2(),
-                                 st->gamma + (threadIdx.x & 3) + 4 * nt, L);
+          [&](int h, int nt, unsigned who) {
+            return exact_product(&at(c ? Y : U, pl.e[h] - (threadIdx.x & 3)), nullptr, double2(), st->gamma + 4 * nt,
+                                 L, who);
           },
           [&](int h, int nt, double2 w, double2 p) {
             if (!pl.ok(h, nt)) return;
