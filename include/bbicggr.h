@@ -321,8 +321,8 @@ int wd_set_link_reals(wd_ctx* ctx, int reals);
  * context allocates at the first product with a given L and grows for a larger one (an outgrown block that a
  * captured product uses is kept until wd_destroy).  When there is no room for the block, or while the
  * stream is being captured before the context's first product, the product runs as with 0; a context whose
- * tables of this form (3.6 KB per site) find no room has form 0, and |kappa| below 2^-6 runs as form 0.  0: every operation on the
- * FP64 pipe.  Asking for 1 with other links, or without the tables, is WD_EINVAL.  wd_get_apply_form
+ * tables of this form (3.6 KB per site) find no room has form 0, and |kappa| below 2^-6 runs as form 0.
+ * 0: every operation on the FP64 pipe.  Asking for 1 with other links, or without the tables, is WD_EINVAL.  wd_get_apply_form
  * returns the form (-1 for a NULL ctx). */
 int wd_set_apply_form(wd_ctx* ctx, int form);
 int wd_get_apply_form(const wd_ctx* ctx);

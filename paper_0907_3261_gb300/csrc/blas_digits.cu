@@ -408,8 +408,10 @@ __device__ __noinline__ bool add_in_fp64(double2* out, int ld, const double2* A,
   bool lossy = false;
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt) {
-    const unsigned w0 = __shfl_sync(0xFFFFFFFFu, within[2 * mt], g >> 1), w1 = __shfl_sync(0xFFFFFFFFu, within[2 * mt + 1], g >> 1);
-    const unsigned s0 = __shfl_sync(0xFFFFFFFFu, some[2 * mt], g >> 1), s1 = __shfl_sync(0xFFFFFFFFu, some[2 * mt + 1], g >> 1);
+    const unsigned w0 = __shfl_sync(0xFFFFFFFFu, within[2 * mt], g >> 1);
+    const unsigned w1 = __shfl_sync(0xFFFFFFFFu, within[2 * mt + 1], g >> 1);
+    const unsigned s0 = __shfl_sync(0xFFFFFFFFu, some[2 * mt], g >> 1);
+    const unsigned s1 = __shfl_sync(0xFFFFFFFFu, some[2 * mt + 1], g >> 1);
     const unsigned w = (g & 1) ? w1 : w0, s = (g & 1) ? s1 : s0;
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
@@ -529,11 +531,12 @@ struct Gram {
       const unsigned p0 = r0 & r0 >> 1, p1 = r1 & r1 >> 1;
       if (!((p0 & p0 >> 2 | p1 & p1 >> 2) & 0x11111111u)) {
         auto four = [](const int e[NI]) {
-          return make_int4(e[0], NI > 1 ? e[NI > 1 ? 1 : 0] : 0, NI > 2 ? e[NI > 2 ? 2 : 0] : 0, NI > 3 ? e[NI > 3 ? 3 : 0] : 0);
+          return make_int4(e[0], e[NI > 1 ? 1 : 0], e[NI > 2 ? 2 : 0], e[NI > 3 ? 3 : 0]);
         };
         __syncwarp();                      // the warp may have just written the rows
-        if (add_in_fp64(out, LD, reinterpret_cast<const double2*>(pa) + n0 * L, reinterpret_cast<const double2*>(pb) + n0 * L,
-                        (int)min(16LL, n1 - n0), L, four(ea), four(eb), ND == 8 ? 1 : GR_SPAN))
+        const double2 *ra = reinterpret_cast<const double2*>(pa), *rb = reinterpret_cast<const double2*>(pb);
+        if (add_in_fp64(out, LD, ra + n0 * L, rb + n0 * L, (int)min(16LL, n1 - n0), L, four(ea), four(eb),
+                        ND == 8 ? 1 : GR_SPAN))
           return;
       }
     }

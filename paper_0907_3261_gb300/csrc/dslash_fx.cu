@@ -30,8 +30,8 @@
 // components are loaded while the current one is summed.
 //
 // Measured on a GB300, Y = A X with the copy of X into the field form, 16^3x32, L = 12: 0.72 ms (0.10 of
-// it the copy; 0.71 without the sites apart), against 1.51 ms for the same product in exact FP32 sums on fixed grids and 3.09 ms on the
-// FP64 pipe; 4^4, L = 1: 17 us against 61 us (a thread's serial chain is a quarter as long); 32^3x64,
+// it the copy; 0.71 without the sites apart), against 1.51 ms for the same product in exact FP32 sums on
+// fixed grids and 3.09 ms on the FP64 pipe; 4^4, L = 1: 17 us against 61 us (a thread's serial chain is a quarter as long); 32^3x64,
 // L = 12: 11.3 against 23.4 ms; j = 12 FP64 sweeps on 8^3x16, L = 12: 0.57 against 1.63 ms.  Error
 // against quad precision (4^4, Gaussian X): 0.80e-16 of |A X|, against 1.56e-16 in exact FP32 sums with
 // FP64 site blocks; 12 sweeps 2.0e-16 against 2.7e-16.  Bound by the multiplier pipe (about 72% of its

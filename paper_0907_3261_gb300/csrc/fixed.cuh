@@ -14,7 +14,9 @@ typedef unsigned long long u64;
 constexpr int FX_EMIN = 1;                 // smallest exponent of a field made from FP64
 constexpr int FX_NONFINITE = 30000;        // the exponent of a spinor with an infinity or a NaN
 constexpr int FX_EK = -4;                  // smallest exponent of the links' scale
-constexpr int FX_APART = 1;                // bits by which a site's field may exceed its neighbours' before its block is done in FP64
+// Bits by which a site's field may exceed its neighbours' before its block is done in FP64: beyond them the common
+// scale would cost its small components more than FP64's rounding of the neighbours' part.
+constexpr int FX_APART = 1;
 constexpr int TPB = 128;
 constexpr unsigned NB_MASK = (1u << 26) - 1u;
 
